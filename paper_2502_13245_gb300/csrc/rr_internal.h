@@ -287,6 +287,33 @@ rr_status launch_scatter_items(const OutArgs &o, const uint64_t *item_key, const
 rr_status launch_sort_segments(const OutArgs &o, uint64_t *tmp_keys, const int32_t *qlist, int32_t nlist,
                                int64_t max_seg, cudaStream_t s);
 
+// Distribution sort of many results: items (slot, key) of nslots segments into the CSR, sorted per segment.
+struct SlotBins {
+    uint32_t base, nb;        // the slot's bins
+    uint32_t lo, scale;       // bin of distance key dk: base + mulhi(dk - lo, scale)
+};
+struct BinSortArgs {
+    OutArgs o;
+    const uint64_t *item_key;
+    const int32_t *item_slot; // < 0: no item
+    int64_t nitems;
+    const int32_t *qlist;     // slot -> query (nullptr: slot = query)
+    int32_t nslots;
+    const int32_t *slot_count;
+    const uint64_t *lo_keys;  // per query (stride lo_stride): a key at the low end of its results, or
+    int64_t lo_stride;
+    const uint32_t *lo_dk;    // per slot: its smallest distance key
+    const uint32_t *rkey;     // per query: the largest distance key
+    uint64_t *tmp;            // o.total keys
+    // carved from the scratch by launch_bin_sort
+    SlotBins *info;
+    uint32_t *rank, *bin_cnt, *big, *ctr;
+    int64_t *bin_start;
+};
+// end offset of the scratch the sort needs from offset `at` on
+size_t bin_sort_end(int64_t nitems, int64_t nslots, size_t at);
+rr_status launch_bin_sort(BinSortArgs a, uint8_t *base, size_t at, cudaStream_t s);
+
 // Brute force (Def. 2.1): count pass and fill pass over all (query, point) pairs.
 rr_status launch_brute(const SearchArgs &a, int32_t *counts, const int64_t *offsets, int32_t *cursor,
                        uint64_t *keys, int fill, cudaStream_t s, int dtype_code);
