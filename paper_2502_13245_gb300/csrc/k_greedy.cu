@@ -31,6 +31,11 @@ namespace rr {
 
 namespace {
 
+// the bitmap of a slot
+__device__ __forceinline__ int32_t seen_of(const GreedyArgs &g, int32_t slot) {
+    return g.hand_of ? __ldg(g.hand_of + slot) : slot;
+}
+
 template <bool COUNT>
 __global__ void greedy_init_kernel(GreedyArgs g) {
     const int b = g.s.beam;
@@ -61,13 +66,13 @@ __global__ void __launch_bounds__(256) greedy_level_kernel(GreedyArgs g) {
                     (size_t)warp * R;
     const int64_t nw = (int64_t)gridDim.x * wpc;
     for (int64_t it = g.begin + (int64_t)blockIdx.x * wpc + warp; it < g.end; it += nw) {
-        const int32_t slot = g.item_slot[it];
-        const uint32_t p = key_id(g.item_key[it]);
+        const int32_t slot = g.in_slot[it];
+        const uint32_t p = key_id(g.in_key[it]);
         const int32_t qi = g.qlist[slot];
         uint4 q[CPL];
         load_query<CPL>(a, a.queries + (size_t)qi * a.row_stride, q);
         const uint32_t rk = a.rkey[qi];
-        uint32_t *seen = g.seen + (size_t)slot * g.seen_words;
+        uint32_t *seen = g.seen + (size_t)seen_of(g, slot) * g.seen_words;
         // f in N_out(p*) \ V, each evaluated once per query (exact bitmap)
         const uint32_t *row = a.adj + (size_t)p * R;
         int nc = 0;
@@ -172,8 +177,8 @@ __global__ void __launch_bounds__(256) greedy_expand_kernel(GreedyArgs g) {
                 const uint32_t io = x / R;
                 k[u] = x - io * R;
                 const int64_t it = g.begin + io;
-                slot[u] = g.item_slot[it];
-                p[u] = key_id(g.item_key[it]);
+                slot[u] = g.in_slot[it];
+                p[u] = key_id(g.in_key[it]);
             }
         }
 #pragma unroll
@@ -187,7 +192,7 @@ __global__ void __launch_bounds__(256) greedy_expand_kernel(GreedyArgs g) {
             wp[u] = nullptr;
             w[u] = 0xFFFFFFFFu;
             if (j[u] < (uint32_t)a.n) {
-                wp[u] = g.seen + (size_t)slot[u] * g.seen_words + (j[u] >> 5);
+                wp[u] = g.seen + (size_t)seen_of(g, slot[u]) * g.seen_words + (j[u] >> 5);
                 w[u] = *wp[u];  // bits only go from 0 to 1 during the phase: a set bit read here is final
             }
         }
@@ -238,8 +243,8 @@ __global__ void __launch_bounds__(256, 4) greedy_expand_rows_kernel(GreedyArgs g
 #pragma unroll
     for (int i = 0; i < IW; i++) {
         const int64_t it = warp_g * IW + i;
-        slot[i] = it < nitems ? g.item_slot[g.begin + it] : -1;
-        p[i] = it < nitems ? key_id(g.item_key[g.begin + it]) : 0u;
+        slot[i] = it < nitems ? g.in_slot[g.begin + it] : -1;
+        p[i] = it < nitems ? key_id(g.in_key[g.begin + it]) : 0u;
     }
     for (int64_t i0 = warp_g * IW; i0 < nitems; i0 += step) {
         uint32_t j[NP];
@@ -258,8 +263,8 @@ __global__ void __launch_bounds__(256, 4) greedy_expand_rows_kernel(GreedyArgs g
 #pragma unroll
         for (int i = 0; i < IW; i++) {
             const int64_t it = i0 + step + i;
-            nslot[i] = it < nitems ? g.item_slot[g.begin + it] : -1;
-            np[i] = it < nitems ? key_id(g.item_key[g.begin + it]) : 0u;
+            nslot[i] = it < nitems ? g.in_slot[g.begin + it] : -1;
+            np[i] = it < nitems ? key_id(g.in_key[g.begin + it]) : 0u;
         }
         uint32_t w[NP];
         uint32_t *wp[NP];
@@ -269,7 +274,7 @@ __global__ void __launch_bounds__(256, 4) greedy_expand_rows_kernel(GreedyArgs g
             wp[e] = nullptr;
             w[e] = 0xFFFFFFFFu;
             if (j[e] < (uint32_t)a.n) {
-                wp[e] = g.seen + (size_t)slot[i] * g.seen_words + (j[e] >> 5);
+                wp[e] = g.seen + (size_t)seen_of(g, slot[i]) * g.seen_words + (j[e] >> 5);
                 w[e] = *wp[e];  // bits only go from 0 to 1 during the phase: a set bit read here is final
             }
         }

@@ -87,16 +87,17 @@ __global__ void scatter_items_kernel(OutArgs o, const uint64_t *item_key, const 
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~(int64_t)31; base < nitems; base += stride) {
         const int64_t t = base + lane;
-        const bool ok = t < nitems;
-        const int32_t s = ok ? item_slot[t] : -1;
+        const int32_t s = t < nitems ? item_slot[t] : -1;
+        const bool ok = s >= 0;
         const int32_t prev = __shfl_up_sync(0xffffffffu, s, 1);
         const bool head = ok && (lane == 0 || prev != s);
         const unsigned hm = __ballot_sync(0xffffffffu, head);
         int32_t r0 = 0;
+        // a run ends at the next lane of another slot, or of none
+        const unsigned brk = __ballot_sync(0xffffffffu, lane == 0 || prev != s);
         if (head) {
-            const unsigned later = hm & ~((2u << lane) - 1u);
-            const int stop = later ? __ffs(later) - 1 : (nitems - base < 32 ? (int)(nitems - base) : 32);
-            r0 = atomicAdd(cursor + s, stop - lane);
+            const unsigned later = brk & ~((2u << lane) - 1u);
+            r0 = atomicAdd(cursor + s, (later ? __ffs(later) - 1 : 32) - lane);
         }
         // the head of this lane's run: the last head at or before the lane (lane 0 is one when ok)
         const unsigned upto = hm & ((2u << lane) - 1u);

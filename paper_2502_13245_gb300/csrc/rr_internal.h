@@ -78,6 +78,8 @@ struct rr_index {
     rr::Grow dbl_s[2];      // doubling: S of the active queries (double buffered)
     rr::Grow dbl_tmp;       // doubling: sort scratch of S u V
     rr::Grow cand;          // greedy candidate list of a level chunk (8-bit indexes)
+    rr::Grow front;         // greedy frontier lists
+    rr::Grow hand;          // greedy queries handed from the cluster kernel to the two-pass levels
     rr::Grow dbl_seen;      // warm-restart doubling: per-query bitmaps of every id evaluated
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // profile: start, beam, phase2, end
     rr_profile prof = {};
@@ -183,6 +185,9 @@ struct GreedyArgs {
     int64_t seen_words;
     uint64_t *item_key;        // appended in-range results (keys)
     int32_t *item_slot;
+    const uint64_t *in_key;    // the list the level's items [begin, end) are read from: the appended results, or
+    const int32_t *in_slot;    // the pending items of queries handed over by the cluster kernel
+    const int32_t *hand_of;    // handed-over queries: slot -> its bitmap in seen (nullptr: slot = bitmap)
     unsigned long long *tail;  // device append cursor
     int64_t cap;               // item capacity
     int32_t *slot_count;       // results per slot
@@ -194,6 +199,42 @@ struct GreedyArgs {
     unsigned long long *ccount;  // device: candidates appended (zeroed before each chunk)
     int64_t ccap;              // candidate capacity (items per chunk x R)
 };
+
+// Alg. 2 with a cluster of CTAs per query, bitmaps in shared memory (k_bfs.cuh).
+constexpr int kBfsThreads = 768;  // threads of a CTA
+struct BfsShape {
+    int cl_log2, threads, clusters, bm_words;
+    uint32_t fcap;             // entries of one frontier list (two a cluster)
+    size_t smem;
+};
+struct BfsArgs {
+    SearchArgs s;
+    const int32_t *qlist;      // slot -> query
+    const int32_t *np2;        // queued queries
+    int32_t *next, *done, *handed, *overflow, *levels;  // device counters, zero at the start
+    unsigned long long *tail;  // item append cursor, zero at the start
+    uint64_t *item_key;
+    int32_t *item_slot;        // -1: no item
+    int64_t cap;
+    int32_t *slot_count;       // results per slot (so far, for a query handed over)
+    uint32_t *front;           // clusters x 2 x fcap
+    uint32_t fcap;
+    int32_t cl_log2, bm_words;
+    uint32_t bail_total, bail_front;  // a query with this many results and this large a frontier is handed over
+    int32_t bail_slots;               // when at most bail_slots queries are unfinished
+    int32_t hand_cap;          // room for handed-over bitmaps (hand_words each) and pending items
+    uint32_t pend_cap;
+    uint32_t *pend_count;      // zero at the start
+    int32_t *hand_of;
+    uint32_t *hand_bits;
+    int64_t hand_words;
+    uint64_t *pend_key;
+    int32_t *pend_slot;
+};
+// false: the index is too large for the bitmaps, the two-pass levels are the faster ones
+bool bfs_shape(int64_t n, int64_t nq, BfsShape *s);
+size_t bfs_front_bytes(const BfsShape &s);
+rr_status launch_bfs(BfsArgs g, const BfsShape &s, cudaStream_t st, int dtype_code);
 
 rr_status launch_greedy_init(const GreedyArgs &g, cudaStream_t s, int dtype_code);
 rr_status launch_greedy_level(const GreedyArgs &g, cudaStream_t s, int dtype_code);
@@ -281,6 +322,7 @@ struct OutArgs {
 rr_status launch_copy_slots(const OutArgs &o, const uint64_t *keys, int64_t stride, const int32_t *count,
                             const int32_t *qlist, int32_t nlist, cudaStream_t s);
 // scatter items (slot, key) to CSR positions of their queries, then sort each listed segment
+// (slot -1: no item)
 rr_status launch_scatter_items(const OutArgs &o, const uint64_t *item_key, const int32_t *item_slot,
                                int64_t nitems, const int32_t *qlist, int32_t *cursor, uint64_t *tmp_keys,
                                cudaStream_t s);

@@ -16,6 +16,10 @@ namespace {
 
 size_t ru(size_t x) { return (x + 255) & ~size_t(255); }
 
+// device counter words (zeroed before the beam phase): queued queries, status, work queues and the item cursor
+enum { kCtrP2 = 0, kCtrError = 1, kCtrNextQ = 2, kCtrBfsNext = 3, kCtrBfsDone = 4, kCtrHand = 5, kCtrOverflow = 6,
+       kCtrLevels = 7, kCtrTail = 8, kCtrCand = 10, kCtrPend = 12, kCtrWords = 16 };
+
 struct Search {
     rr_index *ix;
     cudaStream_t st;
@@ -28,9 +32,12 @@ struct Search {
     uint8_t *flags = nullptr;   // device flags (result array or arena)
     rr_query_stats *stats_res = nullptr;  // device stats result array (device results)
     // phase-2 per-slot arrays (arena): results per slot, truncation, scatter cursor, item tail
-    int32_t *slot_count = nullptr, *slot_trunc = nullptr, *slot_cursor = nullptr;
+    int32_t *slot_count = nullptr, *slot_trunc = nullptr, *slot_cursor = nullptr, *hand_of = nullptr;
     unsigned long long *tail = nullptr;
+    int32_t *counters = nullptr;
     int32_t phase2_steps = 0;   // greedy levels or doubling rounds run
+    int64_t total = -1;         // results of the last scan of the counts (-1: not scanned since they changed)
+    cudaEvent_t prof_ev = nullptr;  // profiled call: recorded at the end of phase 2
     // result arrays allocated for device results (freed on failure)
     std::vector<void *> owned;
 
@@ -79,7 +86,7 @@ rr_status stage(Search &S, const void *queries, const double *radii, double radi
     need += ru((size_t)nq * 8);                                  // radius keys
     need += ru((size_t)nq * b * 8);                              // beam results
     need += 3 * ru((size_t)nq * 4);                              // counts, queue/cursor, spare
-    need += 3 * ru((size_t)nq * 4) + ru(64);                     // phase-2 slot arrays + tail
+    need += 4 * ru((size_t)nq * 4);                              // phase-2 slot arrays
     need += ru(256);                                             // counters
     need += ru((size_t)nq) + ru((size_t)(nq + 1) * 8);           // flags, offsets (host results)
     need += ru((size_t)nq * sizeof(rr_query_stats));             // stats
@@ -136,6 +143,8 @@ rr_status stage(Search &S, const void *queries, const double *radii, double radi
     int32_t *counters = (int32_t *)A.take(256);
     a.p2_count = counters;
     a.error = counters + 1;
+    S.counters = counters;
+    S.tail = (unsigned long long *)(counters + kCtrTail);
     RR_CUDA(cudaMemsetAsync(counters, 0, 256, S.st));
     uint8_t *flags_a = (uint8_t *)A.take((size_t)std::max<int64_t>(nq, 1));
     int64_t *offs_a = (int64_t *)A.take((size_t)(nq + 1) * 8);
@@ -149,8 +158,8 @@ rr_status stage(Search &S, const void *queries, const double *radii, double radi
     S.slot_count = (int32_t *)A.take((size_t)std::max<int64_t>(nq, 1) * 4);
     S.slot_trunc = (int32_t *)A.take((size_t)std::max<int64_t>(nq, 1) * 4);
     S.slot_cursor = (int32_t *)A.take((size_t)std::max<int64_t>(nq, 1) * 4);
-    S.tail = (unsigned long long *)A.take(64);
-    if (!a.res_count || !offs_a || !stats_a || (stats && !a.count_bits) || !S.tail) {
+    S.hand_of = (int32_t *)A.take((size_t)std::max<int64_t>(nq, 1) * 4);
+    if (!a.res_count || !offs_a || !stats_a || (stats && !a.count_bits) || !S.hand_of) {
         set_error("internal: arena sizing");
         return RR_EINTERNAL;
     }
@@ -177,23 +186,30 @@ rr_status stage(Search &S, const void *queries, const double *radii, double radi
     return RR_OK;
 }
 
-// Scan the final per-query counts, read the total (and the device status), allocate the id/dist arrays.
+// Scan the per-query counts; read the counter words and the total.  hc[0 .. kCtrWords) holds the counters then.
+rr_status scan_counts(Search &S) {
+    rr_status s;
+    if ((s = launch_scan(S.a.res_count, S.nq, S.offsets, S.st)) != RR_OK) return s;
+    RR_CUDA(cudaMemcpyAsync(S.hc, S.counters, kCtrWords * 4, cudaMemcpyDeviceToHost, S.st));
+    RR_CUDA(cudaMemcpyAsync(S.hc + kCtrWords, S.offsets + S.nq, 8, cudaMemcpyDeviceToHost, S.st));
+    RR_CUDA(cudaStreamSynchronize(S.st));
+    memcpy(&S.total, S.hc + kCtrWords, 8);
+    if (S.hc[kCtrError] != 0) {
+        set_error("a device-side guard tripped (code %d)", S.hc[kCtrError]);
+        return RR_EINTERNAL;
+    }
+    return RR_OK;
+}
+
+// Allocate the id/dist arrays for the final per-query counts.
 // extra_keys: also room for total sort keys at the start of the staging buffer; bin_items, bin_slots: and for the
 // bin sort's scratch, at *bin_at.
 rr_status scan_and_alloc(Search &S, int64_t *total, uint32_t **ids, void **dists, size_t extra_keys,
                          int64_t bin_items, int64_t bin_slots, size_t *bin_at) {
     rr_index *ix = S.ix;
     rr_status s;
-    if ((s = launch_scan(S.a.res_count, S.nq, S.offsets, S.st)) != RR_OK) return s;
-    int64_t *ht = (int64_t *)S.hc;
-    RR_CUDA(cudaMemcpyAsync(ht, S.offsets + S.nq, 8, cudaMemcpyDeviceToHost, S.st));
-    RR_CUDA(cudaMemcpyAsync(S.hc + 2, S.a.error, 4, cudaMemcpyDeviceToHost, S.st));
-    RR_CUDA(cudaStreamSynchronize(S.st));
-    *total = ht[0];
-    if (S.hc[2] != 0) {
-        set_error("a device-side guard tripped (code %d)", S.hc[2]);
-        return RR_EINTERNAL;
-    }
+    if (S.total < 0 && (s = scan_counts(S)) != RR_OK) return s;
+    *total = S.total;
     const size_t t = (size_t)std::max<int64_t>(*total, 1);
     if (S.dev) {
         *ids = (uint32_t *)S.res_alloc(t * 4);
@@ -268,56 +284,75 @@ constexpr int64_t kBinSortItems = 8192;
 
 struct GreedyOut {
     int64_t nitems = 0;
-    int32_t *slot_cursor = nullptr;
 };
 
-// Alg. 2 for the np2 queued queries, level by level (see k_greedy.cu).
-rr_status run_greedy(Search &S, int32_t np2, GreedyOut &go) {
+// Queries that the cluster kernel handed to the two-pass levels: their pending items, bitmaps, and the items so far.
+struct HandOver {
+    const uint64_t *key;
+    const int32_t *slot;
+    int64_t count;
+    uint32_t *bits;
+    int64_t tail;
+};
+
+// Alg. 2 level by level (see k_greedy.cu) for the np2 queued queries, or from where the cluster kernel left the
+// handed-over ones.  *capped: an item found no room within max_results_total.
+rr_status run_greedy(Search &S, int32_t np2, const HandOver *ho, GreedyOut &go, bool *capped) {
     rr_index *ix = S.ix;
     const SearchArgs &a = S.a;
     const int b = a.beam;
     const int64_t words = (ix->n + 31) / 32;
     rr_status s;
-    if ((s = grow(ix->phase2, ru((size_t)np2 * words * 4), 0, S.st)) != RR_OK) return s;
     GreedyArgs g;
     memset(&g, 0, sizeof g);
     g.s = a;
     g.ng = np2;
     g.qlist = a.p2_list;
-    g.seen = (uint32_t *)ix->phase2.p;
     g.seen_words = words;
     g.slot_count = S.slot_count;
     g.slot_trunc = S.slot_trunc;
-    go.slot_cursor = S.slot_cursor;
     g.tail = S.tail;
-    RR_CUDA(cudaMemsetAsync(g.seen, 0, (size_t)np2 * words * 4, S.st));
-    RR_CUDA(cudaMemsetAsync(go.slot_cursor, 0, (size_t)np2 * 4, S.st));
-    const int64_t init = (int64_t)np2 * b;
+    const int64_t init = ho ? ho->tail : (int64_t)np2 * b;  // items before the first level
+    if (ho) {
+        g.seen = ho->bits;
+        g.hand_of = S.hand_of;
+        RR_CUDA(cudaMemsetAsync(g.slot_trunc, 0, (size_t)np2 * 4, S.st));
+    } else {
+        if ((s = grow(ix->phase2, ru((size_t)np2 * words * 4), 0, S.st)) != RR_OK) return s;
+        g.seen = (uint32_t *)ix->phase2.p;
+        RR_CUDA(cudaMemsetAsync(g.seen, 0, (size_t)np2 * words * 4, S.st));
+    }
     const int64_t cap_limit = std::max<int64_t>(S.P.max_results_total, init);
-    int64_t want = std::min<int64_t>(cap_limit, std::max<int64_t>(init * 8, (int64_t)1 << 20));
-    if ((s = grow(ix->item_key, (size_t)want * 8, 0, S.st)) != RR_OK) return s;
-    if ((s = grow(ix->item_slot, (size_t)want * 4, 0, S.st)) != RR_OK) return s;
+    const int64_t want = std::min<int64_t>(cap_limit, std::max<int64_t>(ho ? init : init * 8, (int64_t)1 << 20));
+    if ((s = grow(ix->item_key, (size_t)want * 8, ho ? (size_t)init * 8 : 0, S.st)) != RR_OK) return s;
+    if ((s = grow(ix->item_slot, (size_t)want * 4, ho ? (size_t)init * 4 : 0, S.st)) != RR_OK) return s;
     auto refresh = [&]() {
         g.item_key = (uint64_t *)ix->item_key.p;
         g.item_slot = (int32_t *)ix->item_slot.p;
         g.cap = std::min<int64_t>(cap_limit, (int64_t)std::min(ix->item_key.bytes / 8, ix->item_slot.bytes / 4));
     };
     refresh();
-    unsigned long long *ht = (unsigned long long *)(S.hc + 4);
-    *ht = (unsigned long long)init;
-    RR_CUDA(cudaMemcpyAsync(g.tail, ht, 8, cudaMemcpyHostToDevice, S.st));
-    if ((s = launch_greedy_init(g, S.st, ix->dtype)) != RR_OK) return s;
+    unsigned long long *ht = (unsigned long long *)(S.hc + 2 * kCtrWords);
+    if (!ho) {
+        *ht = (unsigned long long)init;
+        RR_CUDA(cudaMemcpyAsync(g.tail, ht, 8, cudaMemcpyHostToDevice, S.st));
+        if ((s = launch_greedy_init(g, S.st, ix->dtype)) != RR_OK) return s;
+    }
     const bool two_pass = greedy_two_pass(ix->dtype) && a.row_chunks <= 32;
-    g.ccount = S.tail + 1;  // the second word of the tail block
-    int64_t begin = 0, end = init, levels = 0;
+    g.ccount = (unsigned long long *)(S.counters + kCtrCand);
+    int64_t begin = 0, end = ho ? ho->count : init, tail = init, levels = 0;
+    bool pending = ho != nullptr;
+    *capped = false;
     while (begin < end) {
-        const int64_t need = end + (end - begin) * (int64_t)ix->R;
+        const int64_t need = tail + (end - begin) * (int64_t)ix->R;
         if (need > g.cap && g.cap < cap_limit) {
             int64_t ncap = std::min<int64_t>(cap_limit, need);
-            if ((s = grow(ix->item_key, (size_t)ncap * 8, (size_t)end * 8, S.st)) != RR_OK) return s;
-            if ((s = grow(ix->item_slot, (size_t)ncap * 4, (size_t)end * 4, S.st)) != RR_OK) return s;
+            if ((s = grow(ix->item_key, (size_t)ncap * 8, (size_t)tail * 8, S.st)) != RR_OK) return s;
+            if ((s = grow(ix->item_slot, (size_t)ncap * 4, (size_t)tail * 4, S.st)) != RR_OK) return s;
             refresh();
         }
+        g.in_key = pending ? ho->key : g.item_key;
+        g.in_slot = pending ? ho->slot : g.item_slot;
         // 8-bit indexes: expand + evaluate passes over a candidate list of at most 2^27 entries (16 bytes
         // each), so a long level runs in chunks of items
         int64_t chunk = end - begin;
@@ -337,18 +372,88 @@ rr_status run_greedy(Search &S, int32_t np2, GreedyOut &go) {
         }
         RR_CUDA(cudaMemcpyAsync(ht, g.tail, 8, cudaMemcpyDeviceToHost, S.st));
         RR_CUDA(cudaStreamSynchronize(S.st));
-        begin = end;
-        end = (int64_t)std::min<unsigned long long>(*ht, (unsigned long long)g.cap);
+        begin = tail;
+        end = tail = (int64_t)std::min<unsigned long long>(*ht, (unsigned long long)g.cap);
+        pending = false;
+        if (*ht > (unsigned long long)g.cap) *capped = true;
         S.phase2_steps++;
         if (++levels > ix->n + 1) {
             set_error("greedy phase: level guard tripped");
             return RR_EINTERNAL;
         }
     }
-    go.nitems = end;
-    RR_CUDA(cudaMemsetAsync(g.slot_count, 0, (size_t)np2 * 4, S.st));
-    if ((s = launch_count_items(g.item_slot, end, g.slot_count, S.st)) != RR_OK) return s;
+    if (ho && *capped) return RR_OK;  // the caller starts over with every query
+    go.nitems = tail;
+    S.total = -1;
+    const int64_t from = ho ? init : 0;
+    if (!ho) RR_CUDA(cudaMemsetAsync(g.slot_count, 0, (size_t)np2 * 4, S.st));
+    if ((s = launch_count_items(g.item_slot + from, tail - from, g.slot_count, S.st)) != RR_OK) return s;
     return launch_set_counts(S.a.res_count, S.flags, a.p2_list, g.slot_count, g.slot_trunc, np2, S.st);
+}
+
+// When the cluster kernel hands a query over: a CTA expands ~3 probes per clock, the two-pass levels ~86 over the
+// chip but at ~30 us of launches and host round trip a level, so it pays for large frontiers of the last queries.
+constexpr uint32_t kHandTotal = 8192, kHandFront = 4096, kPendCap = 1u << 22;
+constexpr int kHandSlots = 24, kHandCap = 32;
+
+// Alg. 2 for the queued queries, a cluster of CTAs each (k_bfs.cuh), and the scan of the final counts; their number
+// is read back only after both.  Queries handed over by the kernel are finished by the two-pass levels.  If the
+// items hit their list's end or max_results_total, all queries are redone by the two-pass levels, which grow the
+// list and cut results at the cap.
+rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go) {
+    rr_index *ix = S.ix;
+    const SearchArgs &a = S.a;
+    const int64_t words = (ix->n + 31) / 32;
+    rr_status s;
+    const int64_t want = std::min<int64_t>(S.P.max_results_total, (int64_t)1 << 22);
+    if ((s = grow(ix->item_key, (size_t)want * 8, 0, S.st)) != RR_OK) return s;
+    if ((s = grow(ix->item_slot, (size_t)want * 4, 0, S.st)) != RR_OK) return s;
+    if ((s = grow(ix->front, bfs_front_bytes(shape), 0, S.st)) != RR_OK) return s;
+    const uint32_t pend_cap = (uint32_t)std::min<int64_t>(kPendCap, kHandCap * ix->n);
+    const size_t off_pk = ru((size_t)kHandCap * words * 4), off_ps = off_pk + ru((size_t)pend_cap * 8);
+    if ((s = grow(ix->hand, off_ps + (size_t)pend_cap * 4, 0, S.st)) != RR_OK) return s;
+    BfsArgs g;
+    memset(&g, 0, sizeof g);
+    g.s = a;
+    g.qlist = a.p2_list;
+    g.np2 = S.counters + kCtrP2;
+    g.next = S.counters + kCtrBfsNext;
+    g.done = S.counters + kCtrBfsDone;
+    g.handed = S.counters + kCtrHand;
+    g.overflow = S.counters + kCtrOverflow;
+    g.levels = S.counters + kCtrLevels;
+    g.pend_count = (uint32_t *)(S.counters + kCtrPend);
+    g.tail = S.tail;
+    g.item_key = (uint64_t *)ix->item_key.p;
+    g.item_slot = (int32_t *)ix->item_slot.p;
+    g.cap = std::min<int64_t>(S.P.max_results_total, (int64_t)std::min(ix->item_key.bytes / 8, ix->item_slot.bytes / 4));
+    g.slot_count = S.slot_count;
+    g.front = (uint32_t *)ix->front.p;
+    g.bail_total = kHandTotal;
+    g.bail_front = kHandFront;
+    g.bail_slots = kHandSlots >> shape.cl_log2;
+    g.hand_cap = kHandCap;
+    g.pend_cap = pend_cap;
+    g.hand_of = S.hand_of;
+    g.hand_bits = (uint32_t *)ix->hand.p;
+    g.hand_words = words;
+    g.pend_key = (uint64_t *)((uint8_t *)ix->hand.p + off_pk);
+    g.pend_slot = (int32_t *)((uint8_t *)ix->hand.p + off_ps);
+    if ((s = launch_bfs(g, shape, S.st, ix->dtype)) != RR_OK) return s;
+    if (S.prof_ev) RR_CUDA(cudaEventRecord(S.prof_ev, S.st));
+    if ((s = scan_counts(S)) != RR_OK) return s;
+    *np2 = S.hc[kCtrP2];
+    S.phase2_steps = S.hc[kCtrLevels];
+    unsigned long long tail;
+    memcpy(&tail, S.hc + kCtrTail, 8);
+    bool capped = S.hc[kCtrOverflow] != 0 || (int64_t)tail > g.cap;
+    go.nitems = (int64_t)tail;
+    if (!capped && S.hc[kCtrHand] > 0) {
+        const HandOver ho{g.pend_key, g.pend_slot, (int64_t)(uint32_t)S.hc[kCtrPend], g.hand_bits, (int64_t)tail};
+        if ((s = run_greedy(S, *np2, &ho, go, &capped)) != RR_OK) return s;
+    }
+    if (capped && (s = run_greedy(S, *np2, nullptr, go, &capped)) != RR_OK) return s;
+    return RR_OK;
 }
 
 // Alg. 3 for the np2 queued queries: host-driven rounds over the still active ones.
@@ -358,13 +463,11 @@ rr_status run_doubling(Search &S, int32_t np2, GreedyOut &go, bool warm) {
     const int64_t words = (ix->n + 31) / 32;
     const int b_max = S.P.b_max;
     rr_status s;
-    go.slot_cursor = S.slot_cursor;
     if (warm) {
         // warm restart: one bitmap per query of every id it has evaluated, kept across the rounds
         if ((s = grow(ix->dbl_seen, ru((size_t)np2 * words * 4), 0, S.st)) != RR_OK) return s;
         if ((s = launch_zero_words((uint32_t *)ix->dbl_seen.p, (int64_t)np2 * words, S.st)) != RR_OK) return s;
     }
-    RR_CUDA(cudaMemsetAsync(S.slot_cursor, 0, (size_t)np2 * 4, S.st));
     RR_CUDA(cudaMemsetAsync(S.slot_trunc, 0, (size_t)np2 * 4, S.st));
     RR_CUDA(cudaMemsetAsync(S.tail, 0, 8, S.st));
     std::vector<int32_t> act((size_t)np2);
@@ -591,19 +694,26 @@ extern "C" rr_status rr_range_search(rr_index *ix, const void *queries, int64_t 
     if (prof) RR_CUDA(cudaEventRecord(ix->ev[1], S.st));
 
     int32_t np2 = 0;
-    if (a.phase2 && nq > 0) {
+    GreedyOut go;
+    if (prof) S.prof_ev = ix->ev[2];
+    // exact counters are kept by the two-pass levels only
+    BfsShape shape;
+    const bool bfs = greedy && nq > 0 && !a.stats && bfs_shape(ix->n, nq, &shape);
+    if (bfs) {
+        if ((s = run_bfs(S, shape, &np2, go)) != RR_OK) return S.fail(s);
+    } else if (a.phase2 && nq > 0) {
         RR_CUDA(cudaMemcpyAsync(S.hc, a.p2_count, 4, cudaMemcpyDeviceToHost, S.st));
         RR_CUDA(cudaStreamSynchronize(S.st));
         np2 = S.hc[0];
     }
-    GreedyOut go;
-    if (greedy && np2 > 0) {
-        if ((s = run_greedy(S, np2, go)) != RR_OK) return S.fail(s);
+    if (greedy && !bfs && np2 > 0) {
+        bool capped;
+        if ((s = run_greedy(S, np2, nullptr, go, &capped)) != RR_OK) return S.fail(s);
     }
     if (doubling && np2 > 0) {
         if ((s = run_doubling(S, np2, go, warm)) != RR_OK) return S.fail(s);
     }
-    if (prof) RR_CUDA(cudaEventRecord(ix->ev[2], S.st));
+    if (prof && (!bfs || S.total < 0)) RR_CUDA(cudaEventRecord(ix->ev[2], S.st));
     int64_t total = 0;
     uint32_t *ids = nullptr;
     void *dists = nullptr;
@@ -631,8 +741,9 @@ extern "C" rr_status rr_range_search(rr_index *ix, const void *queries, int64_t 
         if ((s = launch_bin_sort(bs, (uint8_t *)ix->outbuf.p, bin_at, S.st)) != RR_OK) return S.fail(s);
     } else if (items) {
         uint64_t *tmp = (uint64_t *)ix->outbuf.p;
+        RR_CUDA(cudaMemsetAsync(S.slot_cursor, 0, (size_t)np2 * 4, S.st));
         if ((s = launch_scatter_items(o, (const uint64_t *)ix->item_key.p, (const int32_t *)ix->item_slot.p, go.nitems,
-                                      a.p2_list, go.slot_cursor, tmp, S.st)) != RR_OK)
+                                      a.p2_list, S.slot_cursor, tmp, S.st)) != RR_OK)
             return S.fail(s);
         if ((s = launch_sort_segments(o, tmp, a.p2_list, np2, 0, S.st)) != RR_OK) return S.fail(s);
     }
