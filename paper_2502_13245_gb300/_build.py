@@ -15,7 +15,7 @@ LIB = os.path.join(HERE, "librr.so")
 
 SOURCES = ["rr_runtime.cu", "rr_search.cu", "k_beam.cu", "k_greedy.cu", "k_doubling.cu", "k_output.cu", "k_brute.cu",
            "k_noalloc.cu", "k_lowp.cu", "rr_serve.cu", "k_build.cu", "k_relabel.cu", "k_bfs_u8.cu", "k_bfs_i8.cu", "k_bfs_f32.cu",
-           "k_bfs_f32_wide.cu"]
+           "k_bfs_f32_wide.cu", "k_brute_tc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]

@@ -104,7 +104,7 @@ __global__ void scatter_items_kernel(OutArgs o, const uint64_t *item_key, const 
         const int h = upto ? 31 - __clz(upto) : 0;
         r0 = __shfl_sync(0xffffffffu, r0, h);
         if (!ok) continue;
-        const int64_t q = qlist[s];
+        const int64_t q = qlist ? qlist[s] : s;
         const int64_t pos = o.offsets[q] + r0 + (lane - h);
         if (pos < 0 || pos >= o.offsets[q + 1]) {
             atomicExch(o.error, 4);
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(1024) sort_segments_kernel(OutArgs o, uint64_t
     extern __shared__ __align__(16) uint8_t smem_raw[];
     uint64_t *sk = reinterpret_cast<uint64_t *>(smem_raw);
     for (int32_t s = blockIdx.x; s < nlist; s += gridDim.x) {
-        int64_t q = qlist[s];
+        int64_t q = qlist ? qlist[s] : s;
         int64_t off = o.offsets[q];
         int m = (int)(o.offsets[q + 1] - off);
         if (m <= 0) continue;

@@ -359,6 +359,11 @@ rr_status launch_bin_sort(BinSortArgs a, uint8_t *base, size_t at, cudaStream_t 
 // Brute force (Def. 2.1): count pass and fill pass over all (query, point) pairs.
 rr_status launch_brute(const SearchArgs &a, int32_t *counts, const int64_t *offsets, int32_t *cursor,
                        uint64_t *keys, int fill, cudaStream_t s, int dtype_code);
+// 8-bit indexes: one pass on the tensor cores; matches are appended to the item list as (query, key), counted per
+// query, and the smallest distance key of each query is taken (k_brute_tc.cu)
+bool brute_tc(int dtype_code);
+rr_status launch_brute_tc(const SearchArgs &a, int32_t *counts, uint32_t *lo_dk, uint64_t *item_key, int32_t *item_slot,
+                          int64_t cap, unsigned long long *tail, cudaStream_t s, int dtype_code);
 // after the greedy levels: slot_count[s] += the items of slot s among items [0, n)
 rr_status launch_count_items(const int32_t *item_slot, int64_t n, int32_t *slot_count, cudaStream_t s);
 // after phase 2: res_count[qlist[s]] = slot_count[s]; truncated slots flag their query

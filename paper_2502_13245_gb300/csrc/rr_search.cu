@@ -762,6 +762,59 @@ extern "C" rr_status rr_range_search(rr_index *ix, const void *queries, int64_t 
     return RR_OK;
 }
 
+// Def. 2.1 for an 8-bit index (k_brute_tc.cu): one pass over all pairs into the item list, then the bin sort.  A list
+// that was too small is grown to the counted total and the pass repeated.
+static rr_status brute_8bit(Search &S, rr_result *out) {
+    rr_index *ix = S.ix;
+    SearchArgs &a = S.a;
+    const int64_t nq = S.nq;
+    uint32_t *lo = (uint32_t *)S.slot_trunc;
+    rr_status s;
+    int64_t want = (int64_t)1 << 20;
+    for (;;) {
+        if ((s = grow(ix->item_key, (size_t)want * 8, 0, S.st)) != RR_OK) return s;
+        if ((s = grow(ix->item_slot, (size_t)want * 4, 0, S.st)) != RR_OK) return s;
+        const int64_t cap = (int64_t)std::min(ix->item_key.bytes / 8, ix->item_slot.bytes / 4);
+        RR_CUDA(cudaMemsetAsync(lo, 0xFF, (size_t)nq * 4, S.st));
+        if ((s = launch_brute_tc(a, a.res_count, lo, (uint64_t *)ix->item_key.p, (int32_t *)ix->item_slot.p, cap, S.tail,
+                                 S.st, ix->dtype)) != RR_OK)
+            return s;
+        if ((s = scan_counts(S)) != RR_OK) return s;
+        if (S.total <= cap) break;
+        want = S.total;
+        RR_CUDA(cudaMemsetAsync(a.res_count, 0, (size_t)nq * 4, S.st));
+        RR_CUDA(cudaMemsetAsync(S.tail, 0, 8, S.st));
+    }
+    int64_t total = 0;
+    uint32_t *ids = nullptr;
+    void *dists = nullptr;
+    size_t bin_at = 0;
+    const bool bins = S.total >= kBinSortItems;
+    if ((s = scan_and_alloc(S, &total, &ids, &dists, 1, bins ? S.total : 0, nq, &bin_at)) != RR_OK) return s;
+    const OutArgs o{nq, S.offsets, 0, ids, dists, S.flags, total, a.error, nullptr};
+    if (!bins) {
+        uint64_t *tmp = (uint64_t *)ix->outbuf.p;  // a.p2_list (zeroed) is the cursor of each segment
+        if ((s = launch_scatter_items(o, (const uint64_t *)ix->item_key.p, (const int32_t *)ix->item_slot.p, total, nullptr,
+                                      a.p2_list, tmp, S.st)) != RR_OK)
+            return s;
+        if (total > 0 && (s = launch_sort_segments(o, tmp, nullptr, (int32_t)nq, 0, S.st)) != RR_OK) return s;
+        return deliver(S, total, ids, dists, out);
+    }
+    BinSortArgs bs;
+    memset(&bs, 0, sizeof bs);
+    bs.o = o;
+    bs.item_key = (const uint64_t *)ix->item_key.p;
+    bs.item_slot = (const int32_t *)ix->item_slot.p;
+    bs.nitems = total;
+    bs.nslots = (int32_t)nq;
+    bs.slot_count = a.res_count;
+    bs.lo_dk = lo;
+    bs.rkey = a.rkey;
+    bs.tmp = (uint64_t *)ix->outbuf.p;
+    if ((s = launch_bin_sort(bs, (uint8_t *)ix->outbuf.p, bin_at, S.st)) != RR_OK) return s;
+    return deliver(S, total, ids, dists, out);
+}
+
 extern "C" rr_status rr_brute_force(rr_index *ix, const void *queries, int64_t nq, const double *radii, double radius,
                                     void *stream, int32_t result_on_device, rr_result *out) {
     if (!out) { set_error("rr_brute_force: out is NULL"); return RR_EINVAL; }
@@ -780,6 +833,10 @@ extern "C" rr_status rr_brute_force(rr_index *ix, const void *queries, int64_t n
     if (s != RR_OK) return S.fail(s);
     SearchArgs &a = S.a;
     a.ext = ix->ext;  // keys carry the caller's ids, so the sort below is by (distance, id)
+    if (nq > 0 && brute_tc(ix->dtype)) {
+        s = brute_8bit(S, out);
+        return s == RR_OK ? RR_OK : S.fail(s);
+    }
     int32_t *counts = a.res_count, *cursor = a.p2_list;
     if ((s = launch_brute(a, counts, nullptr, nullptr, nullptr, 0, S.st, ix->dtype)) != RR_OK) return S.fail(s);
     int64_t total = 0;
