@@ -362,6 +362,383 @@ __global__ void __launch_bounds__(128) round_kernel(DoublingRound d) {
     }
 }
 
+// The same round by a CTA per query, for rounds with few active queries: there the time is that of the longest
+// query, a chain of b and more visits in order, each a row, its seen words, the vectors and the merge behind one
+// another (2^15 visits in all for a query with 10^4 results).  Looking ahead shortens the chain: the next K
+// unvisited keys of the beam are known, so their rows are read and their unseen neighbours evaluated together, a
+// warp (or, with K below the warps, several) per parent.  Parent k is then visited in this step exactly if no
+// neighbour found under the parents before it is as close as it is: the beam's order up to it, and so every choice
+// of Alg. 1, is that of one visit at a time (later keys enter behind it, and a key stays in the beam while fewer
+// than b are below it).  The rest were evaluated for nothing and stay unmarked.  K grows while all of it holds.
+// Measured (GB300, 41 doubling queries of 10^6 x 128 u8, 10 rounds up to b = 8,192, 41 K results): 45.2 -> 16.2 ms.
+// Bound: still the longest query's chain of steps, each about five dependent memory round trips and barriers.
+constexpr int CW = 8;  // warps, and the most parents of a step
+
+// (key | 1) of rank b-1 of M u I and the number of keys of I up to it, as kth_or1, with a warp (32 probes a step)
+__device__ uint64_t warp_kth_or1(const uint64_t *M, int nM, const uint64_t *I, int nI, int b, int *jI) {
+    *jI = nI;
+    if (nM + nI < b) return kEmpty;
+    int lo = max(0, b - nI), hi = min(b, nM);
+    while (lo < hi) {
+        const int step = (hi - lo + 31) >> 5;
+        const int mid = lo + (lane_id() + 1) * step;
+        const bool ok = mid <= hi && ((b - mid >= nI) || ((M[mid - 1] | 1ull) < (I[b - mid] | 1ull)));
+        const int c = __popc(__ballot_sync(0xffffffffu, ok));  // ok falls once
+        lo += c * step;
+        hi = min(hi, lo + step - 1);
+    }
+    const int i = lo, j = b - lo;
+    const uint64_t x = i > 0 ? (M[i - 1] | 1ull) : 0ull;
+    const uint64_t y = j > 0 ? (I[j - 1] | 1ull) : 0ull;
+    *jI = j;
+    return x > y ? x : y;
+}
+
+__host__ __device__ inline int cta_buffer_keys(int R) { return CW * R < 256 ? 256 : CW * R; }
+__host__ __device__ inline size_t round_cta_smem_bytes(int R) {
+    return (size_t)2 * cta_buffer_keys(R) * 8 + (size_t)CW * R * (8 + 8 + 4);
+}
+
+template <int DT, int CPL>
+__global__ void __launch_bounds__(32 * CW) round_cta_kernel(DoublingRound d) {
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    constexpr int UN = CPL == 1 ? 8 : (CPL == 2 ? 4 : 2);
+    __shared__ uint64_t pkey[CW], selk[2 * CW], s_tau;
+    __shared__ int ppos[CW], selp[2 * CW];
+    __shared__ uint32_t mind[CW];
+    __shared__ int s_K, s_nI, s_ns[2], s_evals, s_distinct, s_end, s_cnt;
+    __shared__ unsigned long long s_base;
+    __shared__ int s_nev;
+    const SearchArgs &a = d.s;
+    const int lane = lane_id(), warp = threadIdx.x >> 5, tid = threadIdx.x, T = 32 * CW;
+    const int64_t i = blockIdx.x;
+    const int R = a.R, b = a.beam, ki = cta_buffer_keys(R);
+    uint64_t *I = reinterpret_cast<uint64_t *>(smem_raw), *I2 = I + ki;
+    uint64_t *ckeys = I2 + ki, *skey = ckeys + CW * R;
+    uint64_t *ckey = ckeys + warp * R;
+    uint32_t *cid = reinterpret_cast<uint32_t *>(skey + CW * R) + warp * R;
+
+    const int32_t slot = d.act[i];
+    const int32_t qi = d.qlist[slot];
+    constexpr bool LP = is_lowp(DT);
+    uint4 q[CPL];
+    float qf[16];
+    float qn2 = 0.f;
+    if constexpr (LP) {
+        load_query_lp<DT>(a, reinterpret_cast<const float *>(a.queries + (size_t)qi * a.row_stride), qf);
+        qn2 = query_norm2_lp(a, qf);
+    } else {
+        load_query<CPL>(a, a.queries + (size_t)qi * a.row_stride, q);
+    }
+    const uint32_t rk = a.rkey[qi], ek = a.eskey[qi];
+    const uint32_t rks = LP ? slack_key(a, rk, qn2) : rk;  // approximate keys above rks are out of range
+    uint64_t *M = d.bA + (size_t)i * b;
+    uint64_t *M2 = d.bB + (size_t)i * b;
+    uint64_t *V = d.v + (size_t)i * d.v_cap;
+    uint32_t *seen = d.seen + (size_t)(d.warm ? slot : i) * d.seen_words;
+    uint64_t *EV = d.warm ? d.ev + (size_t)i * d.ev_cap : nullptr;
+    uint32_t *cbits = a.count_bits ? a.count_bits + (size_t)qi * a.words_per_q : nullptr;
+
+    // B <- top-b(S), as in round_kernel
+    int nM;
+    if (d.first) {
+        uint32_t dk0;
+        if constexpr (LP) dk0 = eval_one_lp<DT>(a, qf, qn2, a.start);
+        else dk0 = eval_one<DT, CPL>(a, q, a.start);
+        if (tid == 0) {
+            M[0] = make_key(dk0, a.start);
+            mark_bit(seen, a.start);
+            if (EV) EV[0] = make_key(dk0, a.start);
+        }
+        nM = 1;
+    } else {
+        nM = min(b, d.s_cnt[i]);
+        const uint64_t *S = d.s_old + (size_t)i * d.s_cap;
+        for (int t = tid; t < nM; t += T) {
+            const uint64_t k = d.warm ? S[t] : S[t] & ~1ull;
+            M[t] = k;
+            if (!d.warm) mark_bit(seen, key_id(k));
+        }
+    }
+    if (tid == 0) {
+        s_nev = d.first && EV ? 1 : 0;
+        s_evals = d.first ? 1 : 0;
+        s_distinct = 0;
+        s_end = 0;
+    }
+    __syncthreads();
+    int nI = 0, nvis = 0, Kt = 2, ns = 0;
+    int cM = 0, cI = 0;  // warp 0: everything before them is visited
+    uint64_t tau = (nM >= b) ? (M[b - 1] | 1ull) : kEmpty;
+    const int64_t limit = min(d.v_cap, a.iter_limit);
+
+    // M <- top-b(M u I), I empty
+    auto flush = [&]() {
+        for (int t = tid; t < nM; t += T) {
+            const uint64_t k = M[t];
+            const int pos = t + lb_or1(I, nI, k | 1ull);
+            if (pos < b) M2[pos] = k;
+        }
+        for (int t = tid; t < nI; t += T) {
+            const uint64_t k = I[t];
+            const int pos = t + lb_or1(M, nM, k | 1ull);
+            if (pos < b) M2[pos] = k;
+        }
+        if (warp == 0) {
+            const int pM = cM < nM ? cM + lb_or1(I, nI, M[cM] | 1ull) : 0x7fffffff;
+            const int pI = cI < nI ? cI + lb_or1(M, nM, I[cI] | 1ull) : 0x7fffffff;
+            cM = min(pM, pI);
+            cI = 0;
+        }
+        __syncthreads();
+        nM = min(b, nM + nI);
+        if (warp == 0) cM = min(cM, nM);
+        nI = 0;
+        uint64_t *t = M;
+        M = M2;
+        M2 = t;
+    };
+    // the first n unvisited keys of L[c..nL) up to tau with their positions; c moves to the first (warp 0)
+    auto pick = [&](const uint64_t *L, int nL, int &c, int n, uint64_t *ok, int *op) {
+        int got = 0;
+        for (int t0 = c; t0 < nL && got < n; t0 += 32) {
+            const int t = t0 + lane;
+            const uint64_t k = t < nL ? L[t] : kEmpty;
+            const bool un = t < nL && !(k & 1ull);
+            const unsigned m = __ballot_sync(0xffffffffu, un);
+            if (got == 0) c = m ? t0 + __ffs(m) - 1 : min(t0 + 32, nL);
+            const int r = got + __popc(m & lanemask_lt());
+            if (un && r < n) {
+                ok[r] = k;
+                op[r] = t;
+            }
+            got = min(n, got + __popc(m));
+            if ((__shfl_sync(0xffffffffu, k, 31) | 1ull) > tau) break;
+        }
+        return got;
+    };
+
+    for (int it = 0;; it ^= 1) {
+        if (warp == 0) {
+            if (ns > 0) {
+                int j;
+                tau = warp_kth_or1(M, nM, I, nI, b, &j);
+                nI = j;
+                cI = min(cI, nI);
+            }
+            // the next parents: the Kt smallest unvisited keys of the beam
+            const int gM = pick(M, nM, cM, Kt, selk, selp);
+            const int gI = pick(I, nI, cI, Kt, selk + CW, selp + CW);
+            __syncwarp();
+            const bool inM = lane < gM, inI = lane >= CW && lane < CW + gI;
+            bool use = false;
+            if (inM || inI) {
+                const uint64_t k = selk[lane];
+                const uint64_t *o = inM ? selk + CW : selk;
+                const int no = inM ? gI : gM;
+                int r = inM ? lane : lane - CW;
+                for (int t = 0; t < no; t++) r += o[t] < k;
+                use = r < Kt && (k | 1ull) <= tau;
+                if (use) {
+                    pkey[r] = k;
+                    ppos[r] = inM ? selp[lane] : -1 - selp[lane];
+                }
+            }
+            int K = __popc(__ballot_sync(0xffffffffu, use));
+            __syncwarp();
+            if (a.use_es && K > 0) {
+                uint64_t mn = M[0] | 1ull;
+                if (nI > 0 && (I[0] | 1ull) < mn) mn = I[0] | 1ull;
+                const bool fire = lane < K && key_dk(mn) > rks && nvis + lane >= a.es_vl && key_dk(pkey[lane & (CW - 1)]) > ek;
+                const unsigned m = __ballot_sync(0xffffffffu, fire);
+                if (m) K = __ffs(m) - 1;
+                if (K == 0 && lane == 0) s_end = 1;
+            }
+            if (K > 0 && nvis + K > limit) {
+                K = (int)(limit - nvis);
+                if (K == 0 && lane == 0) {
+                    if (nvis >= a.iter_limit) atomicExch(a.error, 2);
+                    else s_end = 2;
+                }
+            }
+            if (lane == 0) {
+                s_K = K;
+                s_tau = tau;
+                s_nI = nI;
+                s_ns[it] = 0;
+            }
+        }
+        __syncthreads();
+        const int K = s_K;
+        if (K == 0) break;
+        tau = s_tau;
+        nI = s_nI;
+        // a group of warps per parent, each a part of its row: the unseen neighbours and their distances
+        const int lg = K <= 1 ? 0 : 32 - __clz(K - 1);   // parents rounded up to 2^lg
+        const int G = CW >> lg, par = warp / G;
+        int nc = 0;
+        if (par < K) {
+            const int part = (R + G - 1) / G, e1 = min(R, (warp % G + 1) * part);
+            const uint32_t *row = a.adj + (size_t)key_id(pkey[par]) * R;
+            for (int e0 = (warp % G) * part; e0 < e1; e0 += 32) {
+                const int e = e0 + lane;
+                const uint32_t j = e < e1 ? __ldg(row + e) : kSent;
+                const bool v = j < (uint32_t)a.n && !((__ldcg(seen + (j >> 5)) >> (j & 31)) & 1u);
+                const unsigned m = __ballot_sync(0xffffffffu, v);
+                if (v) cid[nc + __popc(m & lanemask_lt())] = j;
+                nc += __popc(m);
+            }
+            __syncwarp();
+            uint32_t mn = 0xffffffffu;
+            if (nc > 0) {
+                if constexpr (LP) eval_candidates_lp<DT, DT == DT_FP8 ? 4 : 8>(a, qf, qn2, cid, nc, ckey);
+                else eval_candidates<DT, CPL, UN>(a, q, cid, nc, ckey);
+                __syncwarp();
+                for (int c = lane; c < nc; c += 32) mn = min(mn, key_dk(ckey[c]));
+                mn = __reduce_min_sync(0xffffffffu, mn);
+            }
+            if (lane == 0) mind[warp] = mn;
+        }
+        __syncthreads();
+        int nk = 1;
+        for (uint32_t mn = 0xffffffffu; nk < K; nk++) {
+            for (int w = (nk - 1) * G; w < nk * G; w++) mn = min(mn, mind[w]);
+            if (mn <= key_dk(pkey[nk])) break;
+        }
+        // V <- V u the first nk parents
+        if (warp == 0 && lane < nk) {
+            const int pos = ppos[lane];
+            V[nvis + lane] = pkey[lane] & ~1ull;
+            if (pos >= 0) M[pos] |= 1ull;
+            else I[-1 - pos] |= 1ull;
+        }
+        if (par < nk) {
+            int neu = 0, dd = 0;
+            for (int c0 = 0; c0 < nc; c0 += 32) {
+                const int c = c0 + lane;
+                const uint64_t k = c < nc ? ckey[c] : kEmpty;
+                const bool v = c < nc && mark_bit(seen, key_id(k));
+                const unsigned m = __ballot_sync(0xffffffffu, v);
+                neu += __popc(m);
+                if (EV && m) {
+                    int at = 0;
+                    if (lane == 0) at = atomicAdd(&s_nev, __popc(m));
+                    at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & lanemask_lt());
+                    if (v && at < d.ev_cap) EV[at] = k;
+                }
+                if (cbits && v) dd += mark_bit(cbits, key_id(k));
+                const bool keep = v && (k | 1ull) < tau;
+                const unsigned mk = __ballot_sync(0xffffffffu, keep);
+                if (mk) {
+                    int at = 0;
+                    if (lane == 0) at = atomicAdd(&s_ns[it], __popc(mk));
+                    at = __shfl_sync(0xffffffffu, at, 0);
+                    if (keep) skey[at + __popc(mk & lanemask_lt())] = k;
+                }
+            }
+            if (a.stats) {
+                for (int o = 16; o > 0; o >>= 1) dd += __shfl_xor_sync(0xffffffffu, dd, o);
+                if (lane == 0) {
+                    atomicAdd(&s_evals, neu);
+                    atomicAdd(&s_distinct, dd);
+                }
+            }
+        }
+        __syncthreads();
+        nvis += nk;
+        Kt = nk == K ? min(CW, 2 * nk) : nk + 1;
+        if (EV && s_nev > d.ev_cap) {
+            if (tid == 0) s_end = 2;
+            break;
+        }
+        ns = s_ns[it];
+        if (ns == 0) continue;
+        if (nI + ns > ki) flush();
+        for (int c = tid; c < ns; c += T) {  // sort by rank: distinct keys
+            const uint64_t k = skey[c];
+            int r = 0;
+            for (int t = 0; t < ns; t++) r += skey[t] < k;
+            ckeys[r] = k;
+        }
+        __syncthreads();
+        // I <- I u survivors
+        for (int t = tid; t < nI; t += T) {
+            const uint64_t k = I[t];
+            I2[t + lb_or1(ckeys, ns, k | 1ull)] = k;
+        }
+        for (int t = tid; t < ns; t += T) {
+            const uint64_t k = ckeys[t];
+            I2[t + lb_or1(I, nI, k | 1ull)] = k;
+        }
+        if (warp == 0) cI = min(cI, lb_or1(I, nI, ckeys[0] | 1ull));
+        __syncthreads();
+        nI += ns;
+        uint64_t *t = I;
+        I = I2;
+        I2 = t;
+    }
+    __syncthreads();
+    if (s_nI > 0) {
+        nI = s_nI;
+        flush();
+        __syncthreads();
+    }
+    const bool stopped = s_end == 1, overflow = s_end == 2;
+    // N = {n in B : d <= r}, a prefix of M
+    int cnt = 0;
+    for (int hi = nM; cnt < hi;) {
+        const int mid = (cnt + hi) >> 1;
+        if (key_dk(M[mid]) <= rks) cnt = mid + 1;
+        else hi = mid;
+    }
+    const int pre = cnt;
+    if constexpr (LP) {
+        __syncthreads();
+        if (warp == 0) {
+            const int c = exact_filter_sort<CPL, UN>(a, qi, M, pre, rk, cid, ckey, R);
+            if (lane == 0) s_cnt = c;
+        }
+        __syncthreads();
+        cnt = s_cnt;
+    }
+    const bool cont = !stopped && !overflow && cnt == b && !d.last;
+    if (!cont) {
+        // finished: append N to the result items
+        if (tid == 0) s_base = cnt > 0 ? atomicAdd(d.tail, (unsigned long long)cnt) : 0ull;
+        __syncthreads();
+        const unsigned long long base = s_base, cap = (unsigned long long)d.cap;
+        const int fit = base >= cap ? 0 : (int)min((unsigned long long)cnt, cap - base);
+        for (int t = tid; t < fit; t += T) {
+            d.item_key[base + t] = M[t] & ~1ull;
+            d.item_slot[base + t] = slot;
+        }
+        if (tid == 0) {
+            d.slot_count[slot] = fit;
+            d.slot_trunc[slot] = (fit < cnt || overflow || (d.last && cnt == b && !stopped)) ? 1 : 0;
+        }
+    }
+    if (tid == 0) {
+        d.status[i] = cont ? 1 : 0;
+        d.nv[i] = nvis;
+        if (d.nev) d.nev[i] = s_nev;
+        if (a.stats) {
+            rr_query_stats *st = a.stats + qi;
+            const int evals = s_evals + (LP ? pre : 0);
+            if (d.first) {
+                st->visits_beam = nvis;
+                st->rounds = 1;
+                st->evals = evals;
+            } else {
+                st->visits_beam += nvis;
+                st->rounds += 1;
+                st->evals += evals;
+                st->distinct += s_distinct;
+            }
+            st->final_beam = b;
+        }
+    }
+}
+
 // CTA per continuing slot: S_new <- the s_cap_new smallest distinct keys of S_old u V.
 __global__ void __launch_bounds__(1024) supdate_kernel(DoublingSUpdate u, int smem_cap) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -433,8 +810,21 @@ __global__ void zero_words_kernel(uint32_t *p, int64_t n) {
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) p[t] = 0;
 }
 
+// Two CTAs of 256 threads (111 registers) fit an SM: up to two waves of them a round goes by CTA.  With more active
+// queries a warp each fills the chip, and the evaluations made for nothing would cost throughput.
+constexpr int kCtaRounds = 608;
+
 template <int DT, int CPL>
 rr_status round_t(const DoublingRound &d, cudaStream_t st) {
+    if (d.na <= kCtaRounds) {
+        const size_t smem = round_cta_smem_bytes(d.s.R);
+        auto k = round_cta_kernel<DT, CPL>;
+        RR_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k<<<(unsigned)d.na, 32 * CW, smem, st>>>(d);
+        RR_CUDA(cudaGetLastError());
+        note_launch();
+        return RR_OK;
+    }
     const int wpc = 4;
     size_t smem = (size_t)wpc * round_smem_bytes(d.s.R);
     auto k = round_kernel<DT, CPL>;
