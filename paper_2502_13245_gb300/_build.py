@@ -13,7 +13,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "librr.so")
 
-SOURCES = ["rr_runtime.cu", "rr_search.cu", "k_beam.cu", "k_greedy.cu", "k_doubling.cu", "k_output.cu", "k_brute.cu",
+SOURCES = ["rr_runtime.cu", "rr_search.cu", "k_beam.cu", "k_beam_cta.cu", "k_greedy.cu", "k_doubling.cu", "k_output.cu", "k_brute.cu",
            "k_noalloc.cu", "k_lowp.cu", "rr_serve.cu", "k_build.cu", "k_relabel.cu", "k_bfs_u8.cu", "k_bfs_i8.cu", "k_bfs_f32.cu",
            "k_bfs_f32_wide.cu", "k_brute_tc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -171,6 +171,10 @@ struct SearchArgs {
 rr_status ensure_lowp(rr_index *ix, int prec, cudaStream_t st);
 void slack_coefficients(const rr_index *ix, int prec, float *A, float *Bq, float *C);
 
+// k_beam_cta.cu
+constexpr int64_t kBeamCta8 = 304, kBeamCta4 = 608, kBeamCta2 = 1216;  // most queries with 8, 4, 2 warps each
+bool beam_cta(const SearchArgs &a);
+rr_status launch_beam_cta(const SearchArgs &a, cudaStream_t st, int dtype_code);
 rr_status launch_beam(const SearchArgs &a, int warps_per_cta, cudaStream_t s, int dtype_code);
 // Alg. 1 without early stop or range filter for graph construction: the queries are stored rows
 // (a.qids), the visits are recorded (a.vis_out); 8-bit indexes only
