@@ -445,21 +445,20 @@ void mark_from(const HostGraph &G, uint32_t src, std::vector<uint8_t> &seen, std
     }
 }
 
-// attach every point the start cannot reach (one sweep in id order); returns the points attached
-int64_t repair_once(HostGraph &G, uint32_t start, int L) {
+// attach every point the start cannot reach (one sweep in id order; `seen` marks those it can); returns the points
+// attached.  *dropped: an edge was given up, which may have cut off others; without one the sweep leaves every point
+// reached.
+int64_t repair_once(HostGraph &G, uint32_t start, int L, std::vector<uint8_t> &seen, bool *dropped) {
     const int64_t n = G.n;
     const int R = G.R;
-    std::vector<uint8_t> seen((size_t)n, 0);
     std::vector<uint32_t> queue((size_t)n);
-    std::vector<int32_t> indeg((size_t)n, 0);
+    std::vector<int32_t> indeg;  // counted when a full row first has to give up an edge
     std::vector<uint32_t> stamp((size_t)n, 0);
     const int maxv = 4 * L + 16;
     std::vector<HEnt> beam((size_t)L);
     std::vector<uint32_t> vis((size_t)maxv);
     std::vector<double> vd((size_t)maxv);
-    for (int64_t u = 0; u < n; u++)
-        for (int k = 0; k < G.deg[u]; k++) indeg[G.adj[(size_t)u * R + k]]++;
-    mark_from(G, start, seen, queue);
+    *dropped = false;
     uint32_t tag = 0;
     int64_t attached = 0;
     for (int64_t u = 0; u < n; u++) {
@@ -489,21 +488,28 @@ int64_t repair_once(HostGraph &G, uint32_t start, int L) {
         if (G.deg[v] < R) {
             row[G.deg[v]++] = (uint32_t)u;
         } else {
+            if (indeg.empty()) {
+                indeg.assign((size_t)n, 0);
+                for (int64_t x = 0; x < n; x++)
+                    for (int k = 0; k < G.deg[x]; k++) indeg[G.adj[(size_t)x * R + k]]++;
+            }
             int kk = 0;
             for (int k = 1; k < R; k++)
                 if (indeg[row[k]] > indeg[row[kk]] || (indeg[row[k]] == indeg[row[kk]] && row[k] > row[kk])) kk = k;
             indeg[row[kk]]--;
             row[kk] = (uint32_t)u;
+            *dropped = true;
         }
-        indeg[u]++;
+        if (!indeg.empty()) indeg[u]++;
         attached++;
         mark_from(G, (uint32_t)u, seen, queue);
     }
     return attached;
 }
 
-int64_t count_unreached(const HostGraph &G, uint32_t start) {
-    std::vector<uint8_t> seen((size_t)G.n, 0);
+// marks what the start reaches; returns how many points it does not
+int64_t mark_unreached(const HostGraph &G, uint32_t start, std::vector<uint8_t> &seen) {
+    seen.assign((size_t)G.n, 0);
     std::vector<uint32_t> queue((size_t)G.n);
     mark_from(G, start, seen, queue);
     int64_t miss = 0;
@@ -747,9 +753,11 @@ extern "C" rr_status rr_build_graph(const void *vectors, int64_t n, int32_t d, i
         G.deg[(size_t)u] = k;
     }
     int64_t attached = 0;
-    for (int it = 0; it < 8; it++) {
-        if (count_unreached(G, (uint32_t)start) == 0) break;
-        attached += repair_once(G, (uint32_t)start, L);
+    std::vector<uint8_t> seen;
+    bool again = true;
+    for (int it = 0; it < 8 && again; it++) {
+        if (mark_unreached(G, (uint32_t)start, seen) == 0) break;
+        attached += repair_once(G, (uint32_t)start, L, seen, &again);
     }
     const auto t2 = clk::now();
     if (info) {
