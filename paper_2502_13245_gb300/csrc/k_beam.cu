@@ -43,6 +43,17 @@ __device__ __forceinline__ int lower_bound_or1(const uint64_t *a, int n, uint64_
     return lo;
 }
 
+// the same, at most N - 1; a holds N (a power of two) sorted keys, kEmpty past its end, so
+// that the steps are fixed and need no bounds
+template <int N>
+__device__ __forceinline__ int lower_bound_padded(const uint64_t *a, uint64_t k1) {
+    int pos = 0;
+#pragma unroll
+    for (int s = N / 2; s > 0; s >>= 1)
+        if ((a[pos + s - 1] | 1ull) < k1) pos += s;
+    return pos;
+}
+
 // number of v[t] <= x (v non-decreasing)
 __device__ __forceinline__ int upper_bound_i32(const int32_t *v, int n, int x) {
     int lo = 0, hi = n;
@@ -100,6 +111,11 @@ __global__ void __launch_bounds__(256, kBeamMinBlocks<DT>) beam_kernel(SearchArg
 template <int DT, int CPL, int BMAX, bool COUNT, bool BUILD>
 __device__ __forceinline__ void search_query(const SearchArgs &a, int hlg, int64_t qi, uint8_t *base) {
     constexpr int UN = CPL == 1 ? 8 : (CPL == 2 ? 4 : 2);
+    // A padded beam is searched in fixed steps and shifted by source instead of by destination: fewer instructions a
+    // visit for a few more bytes of spill.  Long beams, whose suffixes are long, gain (10^6 x 128 u8, beam 192, 10^4
+    // queries: 4.67 -> 4.60 ms a batch); short ones lose (2*10^6 x 256 u8, beam 96 with early stop, 2*10^4 queries:
+    // 6.12 -> 6.32 ms).
+    constexpr bool PADDED = BMAX >= 256;
     const int lane = lane_id();
     const int R = a.R;
     const int b = a.beam;
@@ -134,6 +150,8 @@ __device__ __forceinline__ void search_query(const SearchArgs &a, int hlg, int64
     uint32_t *cbits = COUNT ? a.count_bits + (size_t)qi * a.words_per_q : nullptr;
 
     for (int i = lane; i < H; i += 32) hash[i] = kSent;
+    if constexpr (PADDED)
+        for (int i = lane; i < BMAX; i += 32) B[i] = kEmpty;
     // B <- S = {start}
     uint32_t dk0;
     if constexpr (LP) dk0 = eval_one_lp<DT>(a, qf, qn2, a.start);
@@ -284,8 +302,13 @@ __device__ __forceinline__ void search_query(const SearchArgs &a, int hlg, int64
             bool keep = c < nc && (k | 1ull) < last;
             int lb = 0;
             if (keep) {
-                lb = lower_bound_or1(B, nb, k | 1ull);
-                keep = !(lb < nb && (B[lb] | 1ull) == (k | 1ull));
+                if constexpr (PADDED) {
+                    lb = lower_bound_padded<BMAX>(B, k | 1ull);  // below BMAX: k is under a full B's last key
+                    keep = (B[lb] | 1ull) != (k | 1ull);
+                } else {
+                    lb = lower_bound_or1(B, nb, k | 1ull);
+                    keep = !(lb < nb && (B[lb] | 1ull) == (k | 1ull));
+                }
             }
             unsigned m = __ballot_sync(0xffffffffu, keep);
             if (keep) {
@@ -327,28 +350,49 @@ __device__ __forceinline__ void search_query(const SearchArgs &a, int hlg, int64
         ns = nsu;
         __syncwarp();
         const int lb0 = lbs[0];
-        // B <- top-b(B u survivors): shift the suffix [lb0, nb) right, last chunk first
-        for (int hi = nb; hi > lb0;) {
-            const int lo = max(lb0, hi - 32);
-            const int i = lo + lane;
-            uint64_t k = 0;
-            int dst = b;
-            if (i < hi) {
-                k = B[i];
-                dst = i + upper_bound_i32(lbs, ns, i);
+        // B <- top-b(B u survivors) in place, last chunk first.  posn: the old next entry after its shift
+        int posn = 0x7fffffff;
+        if (PADDED && ns <= 32) {
+            // survivor r goes to lbs[r] + r; any other place x takes the old entry as many places to its left as
+            // there are survivors before x
+            const int lbr = lane < ns ? lbs[lane] : 0x3fffffff;
+            const int pos = lbr + lane;
+            const uint64_t own = lane < ns ? ckey[lane] : 0;
+            const int top = min(b, nb + ns);
+            for (int lo = (top - 1) & ~31; lo + 31 >= lb0; lo -= 32) {
+                const int rel = pos - lo, x = lo + lane;
+                const unsigned m = __reduce_or_sync(0xffffffffu, (unsigned)rel < 32u ? 1u << rel : 0u);
+                const int src = x - __popc(__ballot_sync(0xffffffffu, rel < 0)) - __popc(m & lanemask_lt());
+                const bool mv = x < top && src != x && !((m >> lane) & 1u);
+                const uint64_t k = mv ? B[src] : 0;
+                __syncwarp();
+                if (mv) B[x] = k;
             }
-            __syncwarp();
-            if (dst < b) B[dst] = k;
-            __syncwarp();
-            hi = lo;
-        }
-        for (int c = lane; c < ns; c += 32) {
-            int pos = lbs[c] + c;
-            if (pos < b) B[pos] = ckey[c];
+            if (pos < b) B[pos] = own;
+            if (nxt < nb) posn = nxt + __popc(__ballot_sync(0xffffffffu, lbr <= nxt));
+        } else {
+            for (int hi = nb; hi > lb0;) {
+                const int lo = max(lb0, hi - 32);
+                const int i = lo + lane;
+                uint64_t k = 0;
+                int dst = b;
+                if (i < hi) {
+                    k = B[i];
+                    dst = i + upper_bound_i32(lbs, ns, i);
+                }
+                __syncwarp();
+                if (dst < b) B[dst] = k;
+                __syncwarp();
+                hi = lo;
+            }
+            for (int c = lane; c < ns; c += 32) {
+                int pos = lbs[c] + c;
+                if (pos < b) B[pos] = ckey[c];
+            }
+            if (nxt < nb) posn = nxt + upper_bound_i32(lbs, ns, nxt);
         }
         __syncwarp();
         // first unvisited entry: the smallest survivor, or the old next one after its shift
-        const int posn = nxt < nb ? nxt + upper_bound_i32(lbs, ns, nxt) : 0x7fffffff;
         nb = min(b, nb + ns);
         cur = min(min(posn, lb0), nb);
     }
