@@ -445,6 +445,10 @@ const char *rr_last_error(void);
  *                           a query after L iterations of Alg. 1's loop and
  *                           the call returns RR_EINTERNAL (the guard that
  *                           normally sits at n + 1 iterations); 0 = default
+ *   "brute_wait_tries"      value N >= 0: the waits of the 8-bit exhaustive
+ *                           scan's kernel give up after N tries of about a
+ *                           microsecond and the call returns RR_EINTERNAL (the
+ *                           limit normally is about a second); -1 = default
  * Returns RR_EINVAL for an unknown key. */
 rr_status rr_debug_set(const char *key, int64_t value);
 

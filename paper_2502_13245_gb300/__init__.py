@@ -363,7 +363,8 @@ def beam_hash_lg(beam: int) -> int:
 
 def rr_debug_set(key: str, value: int):
     """Failure-path hooks for tests: "fail_alloc_after" (N-th next device allocation fails; -1 off),
-    "beam_iteration_limit" (per-query iteration guard of the beam / doubling kernels; 0 default)."""
+    "beam_iteration_limit" (per-query iteration guard of the beam / doubling kernels; 0 default),
+    "brute_wait_tries" (tries of a wait in the 8-bit exhaustive scan; -1 default)."""
     _check(load_library().rr_debug_set(key.encode(), int(value)))
 
 

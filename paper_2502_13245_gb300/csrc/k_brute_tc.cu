@@ -38,7 +38,7 @@ constexpr int kM = 128;                    // queries per tile
 constexpr int kEpilogue = 256;             // two groups of four warps, one an accumulator
 constexpr int kProducers = 512;
 constexpr int kThreads = kEpilogue + kProducers + 32;  // and the MMA issuer
-constexpr int kWaits = 1 << 20;            // tries of a wait before it gives up
+constexpr int kWaits = 1 << 20;            // tries of a wait before it gives up (about a second)
 constexpr int kNormRing = 4;               // tiles whose norms are kept (an accumulator may be read while two more tiles load)
 
 __device__ __forceinline__ uint32_t saddr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -57,9 +57,21 @@ __device__ __forceinline__ bool mbar_try(uint64_t *b, uint32_t parity) {
         : "=r"(ok) : "r"(saddr(b)), "r"(parity) : "memory");
     return ok != 0;
 }
-// bounded wait: false when the limit ran out or another role has given up
-__device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity, volatile int *stop) {
-    for (int i = 0; i < kWaits; i++) {
+// Bounded waits: false when `tries` ran out or another role has given up.  A whole warp waits and votes on every
+// try, so that all its lanes leave together, one way or the other: what follows (tcgen05.ld.sync.aligned, full-mask
+// votes) needs the whole warp.  A lane whose try succeeded may try again: the barrier cannot complete two phases
+// further without this warp's own arrival.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *b, uint32_t parity, volatile int *stop, int tries) {
+    for (int i = 0; i < tries; i++) {
+        if (__all_sync(0xffffffffu, mbar_try(b, parity))) return true;
+        if (__any_sync(0xffffffffu, *stop != 0)) return false;
+    }
+    *stop = 1;
+    return false;
+}
+// the same for a single thread
+__device__ __forceinline__ bool mbar_wait_one(uint64_t *b, uint32_t parity, volatile int *stop, int tries) {
+    for (int i = 0; i < tries; i++) {
         if (mbar_try(b, parity)) return true;
         if (*stop) return false;
     }
@@ -117,6 +129,7 @@ struct TcArgs {
     int32_t *item_slot;
     int64_t cap;
     unsigned long long *tail;
+    int32_t wait_tries;  // tries of a wait before it gives up
 };
 
 // 16 stored bytes -> 16 fp16 values of [-128, 127], written as chunks 2c and 2c + 1 of the row; adds the row's
@@ -188,6 +201,7 @@ __global__ void __launch_bounds__(kThreads, 1) brute_tc_kernel(TcArgs g) {
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    __syncwarp();  // the .sync.aligned instructions want the whole warp
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&tmem_base)),
                      "r"(ncols)
@@ -238,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1) brute_tc_kernel(TcArgs g) {
         int it = s;
         for (int64_t tile = t0 + (int64_t)s * g.per_group; tile < g.tiles; tile += 2 * (int64_t)g.per_group, it += 2) {
             const int ring = it % kNormRing;
-            if (!mbar_wait(&tfull[s], (it >> 1) & 1, stop)) break;
+            if (!mbar_wait_warp(&tfull[s], (it >> 1) & 1, stop, g.wait_tries)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int64_t p0 = tile * N;
             for (int c0 = 0; c0 < N; c0 += 32) {
@@ -276,6 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1) brute_tc_kernel(TcArgs g) {
                         cnt++;
                         lo = min(lo, dk);
                     }
+                    __syncwarp();  // before the next load from TMEM
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -305,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, 1) brute_tc_kernel(TcArgs g) {
         int it = 0;
         for (int64_t tile = t0; tile < g.tiles; tile += g.per_group, it++) {
             const int s = it & 1, ring = it % kNormRing;
-            if (it >= 2 && !mbar_wait(&empty[s], ((it >> 1) - 1) & 1, stop)) break;
+            if (it >= 2 && !mbar_wait_warp(&empty[s], ((it >> 1) - 1) & 1, stop, g.wait_tries)) break;
             uint8_t *B = Bt + s * bstage;
 #pragma unroll
             for (int u = 0; u < U; u++) {
@@ -336,8 +351,8 @@ __global__ void __launch_bounds__(kThreads, 1) brute_tc_kernel(TcArgs g) {
         int it = 0;
         for (int64_t tile = t0; tile < g.tiles; tile += g.per_group, it++) {
             const int s = it & 1;
-            if (!mbar_wait(&full[s], (it >> 1) & 1, stop)) break;
-            if (it >= 2 && !mbar_wait(&tempty[s], ((it >> 1) - 1) & 1, stop)) break;
+            if (!mbar_wait_one(&full[s], (it >> 1) & 1, stop, g.wait_tries)) break;
+            if (it >= 2 && !mbar_wait_one(&tempty[s], ((it >> 1) - 1) & 1, stop, g.wait_tries)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             for (int k = 0; k < K / 16; k++) {  // 16 values (32 bytes) a step, 64 a swizzled block
                 const uint32_t ka = abase + (uint32_t)(k >> 2) * kM * 128 + (k & 3) * 32;
@@ -348,14 +363,15 @@ __global__ void __launch_bounds__(kThreads, 1) brute_tc_kernel(TcArgs g) {
             mma_commit(&tfull[s]);
             mbar_arrive(&tfull[s]);
         }
-        if (it >= 1) {
-            // every MMA has read its operands and written its accumulators before the CTA goes on
-            for (int i = 0; i < kWaits && !mbar_try(&empty[(it - 1) & 1], ((it - 1) >> 1) & 1); i++) {}
-        }
+        // every MMA has read its operands and written its accumulators, and every commit has arrived on its barrier,
+        // before the CTA goes on (also when an epilogue group left early)
+        for (int t = it > 2 ? it - 2 : 0; t < it; t++)
+            for (int i = 0; i < kWaits && !(mbar_try(&empty[t & 1], (t >> 1) & 1) && mbar_try(&tfull[t & 1], (t >> 1) & 1)); i++) {}
     }
     __syncwarp();
     __syncthreads();
     if (tid == 0 && stop_flag) atomicExch(a.error, 8);
+    __syncwarp();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
 }
@@ -386,6 +402,7 @@ rr_status launch_brute_tc(const SearchArgs &a, int32_t *counts, uint32_t *lo_dk,
     g.item_slot = item_slot;
     g.cap = cap;
     g.tail = tail;
+    g.wait_tries = brute_wait_tries(kWaits);
     const size_t smem = 1024 + (size_t)kM * k * 2 + 2 * (size_t)g.n_tile * k * 2;
     auto kern = dtype_code == DT_U8 ? brute_tc_kernel<false> : brute_tc_kernel<true>;
     RR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -15,9 +15,11 @@ void note_launch(int k = 1);
 int64_t launches_so_far();
 rr_status cuda_fail(cudaError_t e, const char *what);
 // failure-path hooks set by rr_debug_set: true if this device allocation is to fail;
-// the beam and doubling kernels' per-query iteration guard (default n + 1)
+// the beam and doubling kernels' per-query iteration guard (default n + 1); the tries of a wait in the 8-bit
+// exhaustive scan
 bool inject_alloc_failure();
 int64_t beam_iteration_limit(int64_t n);
+int32_t brute_wait_tries(int32_t def);
 
 #define RR_CUDA(call)                                        \
     do {                                                     \

@@ -40,6 +40,7 @@ rr_status cuda_fail(cudaError_t e, const char *what) {
 // Failure-path hooks (rr_debug_set): process-wide, off by default.
 static std::atomic<int64_t> g_fail_alloc_after{-1};
 static std::atomic<int64_t> g_beam_iteration_limit{0};
+static std::atomic<int64_t> g_brute_wait_tries{-1};
 
 bool inject_alloc_failure() {
     int64_t v = g_fail_alloc_after.load();
@@ -52,6 +53,11 @@ bool inject_alloc_failure() {
 int64_t beam_iteration_limit(int64_t n) {
     const int64_t v = g_beam_iteration_limit.load();
     return v > 0 ? v : n + 1;
+}
+
+int32_t brute_wait_tries(int32_t def) {
+    const int64_t v = g_brute_wait_tries.load();
+    return v >= 0 ? (int32_t)std::min<int64_t>(v, def) : def;
 }
 
 rr_status Arena::reserve(size_t bytes) {
@@ -340,6 +346,10 @@ rr_status rr_debug_set(const char *key, int64_t value) {
     }
     if (!strcmp(key, "beam_iteration_limit")) {
         g_beam_iteration_limit.store(value < 0 ? 0 : value);
+        return RR_OK;
+    }
+    if (!strcmp(key, "brute_wait_tries")) {
+        g_brute_wait_tries.store(value < 0 ? -1 : value);
         return RR_OK;
     }
     set_error("rr_debug_set: unknown key '%s'", key);
