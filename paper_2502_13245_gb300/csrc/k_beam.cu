@@ -444,7 +444,7 @@ template <int DT, int CPL, int BMAX, bool COUNT>
 rr_status launch_k(const SearchArgs &a, int wpc, int hlg, cudaStream_t st) {
     auto k = beam_kernel<DT, CPL, BMAX, COUNT>;
     const size_t smem = (size_t)wpc * warp_smem_bytes(BMAX, a.R * std::max(1, a.expand), hlg);
-    RR_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (rr_status e = allow_smem((const void *)k, smem)) return e;
     int64_t blocks = (a.nq + wpc - 1) / wpc;
     if (a.persistent) {
         int dev = 0, sms = 0, per_sm = 0;
@@ -484,7 +484,7 @@ template <int DT, int BMAX>
 rr_status launch_build_k(const SearchArgs &a, int wpc, int hlg, cudaStream_t st) {
     auto k = beam_kernel<DT, 1, BMAX, false, true>;
     const size_t smem = (size_t)wpc * warp_smem_bytes(BMAX, a.R, hlg);
-    RR_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (rr_status e = allow_smem((const void *)k, smem)) return e;
     const int64_t blocks = (a.nq + wpc - 1) / wpc;
     k<<<(unsigned)blocks, 32 * wpc, smem, st>>>(a, hlg, 0, nullptr);
     RR_CUDA(cudaGetLastError());

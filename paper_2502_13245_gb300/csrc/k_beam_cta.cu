@@ -264,7 +264,7 @@ rr_status launch_t(const SearchArgs &a, cudaStream_t st) {
     auto k = beam_cta_kernel<DT, CPL>;
     const int W = a.nq <= kBeamCta8 ? 8 : (a.nq <= kBeamCta4 ? 4 : 2);
     const size_t smem = cta_smem_bytes(a.beam, a.R, W, kHashLg);
-    RR_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (rr_status e = allow_smem((const void *)k, smem)) return e;
     k<<<(unsigned)a.nq, 32 * W, smem, st>>>(a, kHashLg);
     RR_CUDA(cudaGetLastError());
     note_launch();

@@ -351,7 +351,7 @@ rr_status bfs_r(const BfsArgs &g, const BfsShape &s, cudaStream_t st) {
         cfg.numAttrs = 1;
     }
     auto k = g.cl_log2 == 0 ? bfs_kernel<DT, CPL, RR, false> : bfs_kernel<DT, CPL, RR, true>;
-    RR_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem));
+    if (rr_status e = allow_smem((const void *)k, s.smem)) return e;
     RR_CUDA(cudaLaunchKernelEx(&cfg, k, g));
     note_launch();
     return RR_OK;

@@ -73,15 +73,15 @@ rr_status launch_brute(const SearchArgs &a, int32_t *counts, const int64_t *offs
     size_t smem = (size_t)QT * a.row_chunks * 16;
     switch (dtype_code) {
         case DT_U8:
-            RR_CUDA(cudaFuncSetAttribute(brute_kernel<DT_U8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            if (rr_status e = allow_smem((const void *)brute_kernel<DT_U8>, smem)) return e;
             brute_kernel<DT_U8><<<grid, 256, smem, st>>>(a, counts, offsets, cursor, keys, fill);
             break;
         case DT_I8:
-            RR_CUDA(cudaFuncSetAttribute(brute_kernel<DT_I8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            if (rr_status e = allow_smem((const void *)brute_kernel<DT_I8>, smem)) return e;
             brute_kernel<DT_I8><<<grid, 256, smem, st>>>(a, counts, offsets, cursor, keys, fill);
             break;
         case DT_F32:
-            RR_CUDA(cudaFuncSetAttribute(brute_kernel<DT_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            if (rr_status e = allow_smem((const void *)brute_kernel<DT_F32>, smem)) return e;
             brute_kernel<DT_F32><<<grid, 256, smem, st>>>(a, counts, offsets, cursor, keys, fill);
             break;
         default:

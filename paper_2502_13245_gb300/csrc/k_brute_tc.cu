@@ -405,7 +405,7 @@ rr_status launch_brute_tc(const SearchArgs &a, int32_t *counts, uint32_t *lo_dk,
     g.wait_tries = brute_wait_tries(kWaits);
     const size_t smem = 1024 + (size_t)kM * k * 2 + 2 * (size_t)g.n_tile * k * 2;
     auto kern = dtype_code == DT_U8 ? brute_tc_kernel<false> : brute_tc_kernel<true>;
-    RR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (rr_status e = allow_smem((const void *)kern, smem)) return e;
     kern<<<(unsigned)(groups * g.per_group), kThreads, smem, st>>>(g);
     RR_CUDA(cudaGetLastError());
     note_launch();

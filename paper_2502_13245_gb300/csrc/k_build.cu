@@ -541,7 +541,7 @@ template <int DT>
 rr_status launch_prune(const BuildArgs &b, cudaStream_t st) {
     const int wpc = 4;
     const size_t smem = (size_t)wpc * PruneSmem::bytes(b.mcap, b.s.R);
-    RR_CUDA(cudaFuncSetAttribute(prune_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (rr_status e = allow_smem((const void *)prune_kernel<DT>, smem)) return e;
     prune_kernel<DT><<<(b.nb + wpc - 1) / wpc, 32 * wpc, smem, st>>>(b);
     RR_CUDA(cudaGetLastError());
     note_launch();
@@ -552,7 +552,7 @@ template <int DT>
 rr_status launch_merge(const BuildArgs &b, int32_t nt, cudaStream_t st) {
     const int wpc = 4;
     const size_t smem = (size_t)wpc * PruneSmem::bytes(b.mcap, b.s.R);
-    RR_CUDA(cudaFuncSetAttribute(merge_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (rr_status e = allow_smem((const void *)merge_kernel<DT>, smem)) return e;
     merge_kernel<DT><<<(nt + wpc - 1) / wpc, 32 * wpc, smem, st>>>(b, nt);
     RR_CUDA(cudaGetLastError());
     note_launch();

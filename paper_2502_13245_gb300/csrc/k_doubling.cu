@@ -819,7 +819,7 @@ rr_status round_t(const DoublingRound &d, cudaStream_t st) {
     if (d.na <= kCtaRounds) {
         const size_t smem = round_cta_smem_bytes(d.s.R);
         auto k = round_cta_kernel<DT, CPL>;
-        RR_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (rr_status e = allow_smem((const void *)k, smem)) return e;
         k<<<(unsigned)d.na, 32 * CW, smem, st>>>(d);
         RR_CUDA(cudaGetLastError());
         note_launch();
@@ -828,7 +828,7 @@ rr_status round_t(const DoublingRound &d, cudaStream_t st) {
     const int wpc = 4;
     size_t smem = (size_t)wpc * round_smem_bytes(d.s.R);
     auto k = round_kernel<DT, CPL>;
-    RR_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (rr_status e = allow_smem((const void *)k, smem)) return e;
     k<<<(unsigned)((d.na + wpc - 1) / wpc), 32 * wpc, smem, st>>>(d);
     RR_CUDA(cudaGetLastError());
     note_launch();
@@ -858,7 +858,7 @@ rr_status launch_doubling_supdate(const DoublingSUpdate &u, cudaStream_t st) {
     if (u.nc <= 0) return RR_OK;
     const int smem_cap = 16384;
     size_t smem = (size_t)smem_cap * 8;
-    RR_CUDA(cudaFuncSetAttribute(supdate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (rr_status e = allow_smem((const void *)supdate_kernel, smem)) return e;
     int blocks = u.nc < 152 * 2 ? u.nc : 152 * 2;
     supdate_kernel<<<blocks, 1024, smem, st>>>(u, smem_cap);
     RR_CUDA(cudaGetLastError());

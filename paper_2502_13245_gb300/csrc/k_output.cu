@@ -466,7 +466,7 @@ rr_status launch_bin_sort(BinSortArgs a, uint8_t *base, size_t at, cudaStream_t 
     RR_CUDA(cudaGetDevice(&dev));
     RR_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const int smem_cap = std::max(4096, optin / 8);
-    RR_CUDA(cudaFuncSetAttribute(bin_sort_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_cap * 8));
+    if (rr_status e = allow_smem((const void *)bin_sort_big_kernel, smem_cap * 8)) return e;
     bin_sort_big_kernel<<<(unsigned)std::min<int64_t>(a.nitems / kWarpBin + 1, 152), 1024, (size_t)smem_cap * 8, st>>>(
         a, smem_cap);
     RR_CUDA(cudaGetLastError());
@@ -514,7 +514,7 @@ rr_status launch_sort_segments(const OutArgs &o, uint64_t *tmp, const int32_t *q
     RR_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const int smem_cap = std::max(4096, optin / 8);
     size_t smem = (size_t)smem_cap * 8;
-    RR_CUDA(cudaFuncSetAttribute(sort_segments_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (rr_status e = allow_smem((const void *)sort_segments_kernel, smem)) return e;
     int blocks = nlist < 152 * 2 ? nlist : 152 * 2;
     sort_segments_kernel<<<blocks, 1024, smem, st>>>(o, tmp, qlist, nlist, smem_cap);
     RR_CUDA(cudaGetLastError());

@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <map>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -35,6 +36,31 @@ void set_error(const char *fmt, ...) {
 rr_status cuda_fail(cudaError_t e, const char *what) {
     set_error("%s: %s", what, cudaGetErrorString(e));
     return RR_ECUDA;
+}
+
+rr_status allow_smem(const void *kernel, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void *>, size_t> limit;
+    int dev = 0;
+    RR_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = limit.find({dev, kernel});
+    if (it != limit.end() && bytes <= it->second) return RR_OK;
+    if (it == limit.end()) {
+        try {
+            it = limit.emplace(std::make_pair(dev, kernel), (size_t)0).first;
+        } catch (const std::bad_alloc &) {
+            set_error("host allocation failed");
+            return RR_ENOMEM;
+        }
+    }
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return cuda_fail(e, "cudaFuncSetAttribute(dynamic shared memory)");
+    }
+    it->second = bytes;
+    return RR_OK;
 }
 
 // Failure-path hooks (rr_debug_set): process-wide, off by default.
