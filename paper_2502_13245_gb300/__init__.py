@@ -38,7 +38,7 @@ EXPORTS = ["rr_params_init", "rr_create_index", "rr_load_index", "rr_free_index"
            "rr_range_search", "rr_brute_force", "rr_result_free", "rr_last_error", "rr_last_profile",
            "rr_beam_search_noalloc", "rr_serve_cfg_init", "rr_serve_create", "rr_serve_submit", "rr_serve_poll",
            "rr_serve_collect", "rr_serve_cancel", "rr_serve_stats", "rr_serve_destroy", "rr_result_to_host",
-           "rr_abi_sizes", "rr_debug_set", "rr_build_graph", "rr_index_relabel"]
+           "rr_abi_sizes", "rr_debug_set", "rr_debug_count", "rr_build_graph", "rr_index_relabel"]
 
 
 class RRError(RuntimeError):
@@ -173,6 +173,8 @@ def load_library(path: str | None = None):
     L.rr_serve_destroy.argtypes = [P]
     L.rr_debug_set.restype = ctypes.c_int
     L.rr_debug_set.argtypes = [ctypes.c_char_p, I64]
+    L.rr_debug_count.restype = I64
+    L.rr_debug_count.argtypes = [ctypes.c_char_p]
     L.rr_build_graph.restype = ctypes.c_int
     L.rr_build_graph.argtypes = [P, I64, I32, I32, I32, I32, I32, D, I32, ctypes.c_uint64, I64, I32, P, P]
     _lib = L
@@ -366,6 +368,14 @@ def rr_debug_set(key: str, value: int):
     "beam_iteration_limit" (per-query iteration guard of the beam / doubling kernels; 0 default),
     "brute_wait_tries" (tries of a wait in the 8-bit exhaustive scan; -1 default)."""
     _check(load_library().rr_debug_set(key.encode(), int(value)))
+
+
+def rr_debug_count(key: str) -> int:
+    """How often the library has taken a form of a phase (keys: include/rr.h)."""
+    n = load_library().rr_debug_count(key.encode())
+    if n < 0:
+        raise KeyError(key)
+    return n
 
 
 def rr_last_profile(handle) -> Profile:

@@ -529,7 +529,11 @@ rr_status launch_beam(const SearchArgs &a, int wpc, cudaStream_t st, int dtype_c
         set_error("beam phase: seen-table size 2^%d out of [2^5, 2^14]", hlg);
         return RR_EINVAL;
     }
-    if (beam_cta(a)) return launch_beam_cta(a, st, dtype_code);  // a small batch
+    if (beam_cta(a)) {  // a small batch
+        note_form(kFormBeamCta);
+        return launch_beam_cta(a, st, dtype_code);
+    }
+    note_form(kFormBeamWarp);
     const int cpl = (a.row_chunks + 31) / 32;
     switch (dtype_code) {
         case DT_U8: return launch_b<DT_U8, 1>(a, wpc, hlg, st);

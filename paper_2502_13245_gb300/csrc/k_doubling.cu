@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(32 * CW) round_cta_kernel(DoublingRound d) {
     __shared__ uint64_t pkey[CW], selk[2 * CW], s_tau;
     __shared__ int ppos[CW], selp[2 * CW];
     __shared__ uint32_t mind[CW];
-    __shared__ int s_K, s_nI, s_ns[2], s_evals, s_distinct, s_end, s_cnt;
+    __shared__ int s_K, s_nI, s_ns[2], s_end, s_cnt;
     __shared__ unsigned long long s_base;
     __shared__ int s_nev;
     const SearchArgs &a = d.s;
@@ -437,7 +437,6 @@ __global__ void __launch_bounds__(32 * CW) round_cta_kernel(DoublingRound d) {
     uint64_t *V = d.v + (size_t)i * d.v_cap;
     uint32_t *seen = d.seen + (size_t)(d.warm ? slot : i) * d.seen_words;
     uint64_t *EV = d.warm ? d.ev + (size_t)i * d.ev_cap : nullptr;
-    uint32_t *cbits = a.count_bits ? a.count_bits + (size_t)qi * a.words_per_q : nullptr;
 
     // B <- top-b(S), as in round_kernel
     int nM;
@@ -462,8 +461,6 @@ __global__ void __launch_bounds__(32 * CW) round_cta_kernel(DoublingRound d) {
     }
     if (tid == 0) {
         s_nev = d.first && EV ? 1 : 0;
-        s_evals = d.first ? 1 : 0;
-        s_distinct = 0;
         s_end = 0;
     }
     __syncthreads();
@@ -613,20 +610,17 @@ __global__ void __launch_bounds__(32 * CW) round_cta_kernel(DoublingRound d) {
             else I[-1 - pos] |= 1ull;
         }
         if (par < nk) {
-            int neu = 0, dd = 0;
             for (int c0 = 0; c0 < nc; c0 += 32) {
                 const int c = c0 + lane;
                 const uint64_t k = c < nc ? ckey[c] : kEmpty;
                 const bool v = c < nc && mark_bit(seen, key_id(k));
                 const unsigned m = __ballot_sync(0xffffffffu, v);
-                neu += __popc(m);
                 if (EV && m) {
                     int at = 0;
                     if (lane == 0) at = atomicAdd(&s_nev, __popc(m));
                     at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & lanemask_lt());
                     if (v && at < d.ev_cap) EV[at] = k;
                 }
-                if (cbits && v) dd += mark_bit(cbits, key_id(k));
                 const bool keep = v && (k | 1ull) < tau;
                 const unsigned mk = __ballot_sync(0xffffffffu, keep);
                 if (mk) {
@@ -634,13 +628,6 @@ __global__ void __launch_bounds__(32 * CW) round_cta_kernel(DoublingRound d) {
                     if (lane == 0) at = atomicAdd(&s_ns[it], __popc(mk));
                     at = __shfl_sync(0xffffffffu, at, 0);
                     if (keep) skey[at + __popc(mk & lanemask_lt())] = k;
-                }
-            }
-            if (a.stats) {
-                for (int o = 16; o > 0; o >>= 1) dd += __shfl_xor_sync(0xffffffffu, dd, o);
-                if (lane == 0) {
-                    atomicAdd(&s_evals, neu);
-                    atomicAdd(&s_distinct, dd);
                 }
             }
         }
@@ -691,11 +678,10 @@ __global__ void __launch_bounds__(32 * CW) round_cta_kernel(DoublingRound d) {
         if (key_dk(M[mid]) <= rks) cnt = mid + 1;
         else hi = mid;
     }
-    const int pre = cnt;
     if constexpr (LP) {
         __syncthreads();
         if (warp == 0) {
-            const int c = exact_filter_sort<CPL, UN>(a, qi, M, pre, rk, cid, ckey, R);
+            const int c = exact_filter_sort<CPL, UN>(a, qi, M, cnt, rk, cid, ckey, R);
             if (lane == 0) s_cnt = c;
         }
         __syncthreads();
@@ -721,21 +707,6 @@ __global__ void __launch_bounds__(32 * CW) round_cta_kernel(DoublingRound d) {
         d.status[i] = cont ? 1 : 0;
         d.nv[i] = nvis;
         if (d.nev) d.nev[i] = s_nev;
-        if (a.stats) {
-            rr_query_stats *st = a.stats + qi;
-            const int evals = s_evals + (LP ? pre : 0);
-            if (d.first) {
-                st->visits_beam = nvis;
-                st->rounds = 1;
-                st->evals = evals;
-            } else {
-                st->visits_beam += nvis;
-                st->rounds += 1;
-                st->evals += evals;
-                st->distinct += s_distinct;
-            }
-            st->final_beam = b;
-        }
     }
 }
 
@@ -811,12 +782,14 @@ __global__ void zero_words_kernel(uint32_t *p, int64_t n) {
 }
 
 // Two CTAs of 256 threads (111 registers) fit an SM: up to two waves of them a round goes by CTA.  With more active
-// queries a warp each fills the chip, and the evaluations made for nothing would cost throughput.
+// queries a warp each fills the chip, and the evaluations made for nothing would cost throughput.  Exact counters
+// (stats) are kept by the warp form only: rr_query_stats.evals is what was evaluated, and the lookahead evaluates more.
 constexpr int kCtaRounds = 608;
 
 template <int DT, int CPL>
 rr_status round_t(const DoublingRound &d, cudaStream_t st) {
-    if (d.na <= kCtaRounds) {
+    if (d.na <= kCtaRounds && !d.s.stats) {
+        note_form(kFormRoundCta);
         const size_t smem = round_cta_smem_bytes(d.s.R);
         auto k = round_cta_kernel<DT, CPL>;
         if (rr_status e = allow_smem((const void *)k, smem)) return e;
@@ -825,6 +798,7 @@ rr_status round_t(const DoublingRound &d, cudaStream_t st) {
         note_launch();
         return RR_OK;
     }
+    note_form(kFormRoundWarp);
     const int wpc = 4;
     size_t smem = (size_t)wpc * round_smem_bytes(d.s.R);
     auto k = round_kernel<DT, CPL>;

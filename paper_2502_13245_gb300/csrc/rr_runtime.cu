@@ -68,6 +68,11 @@ static std::atomic<int64_t> g_fail_alloc_after{-1};
 static std::atomic<int64_t> g_beam_iteration_limit{0};
 static std::atomic<int64_t> g_brute_wait_tries{-1};
 
+static std::atomic<int64_t> g_forms[kForms];
+static const char *const kFormKeys[kForms] = {"beam_warp", "beam_cta", "round_warp", "round_cta"};
+
+void note_form(Form f, int64_t k) { g_forms[f].fetch_add(k, std::memory_order_relaxed); }
+
 bool inject_alloc_failure() {
     int64_t v = g_fail_alloc_after.load();
     while (v >= 0) {
@@ -380,6 +385,12 @@ rr_status rr_debug_set(const char *key, int64_t value) {
     }
     set_error("rr_debug_set: unknown key '%s'", key);
     return RR_EINVAL;
+}
+
+int64_t rr_debug_count(const char *key) {
+    for (int f = 0; key && f < kForms; f++)
+        if (!strcmp(key, kFormKeys[f])) return g_forms[f].load(std::memory_order_relaxed);
+    return -1;
 }
 
 void rr_abi_sizes(int64_t out[8]) {

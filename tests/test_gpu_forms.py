@@ -1,0 +1,66 @@
+"""Which form of a phase a call takes (rr_debug_count), and each form against the CPU oracle, bit for bit, at the sizes
+where the other one is the library's choice next door."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rr():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for -m gpu tests")
+    import paper_2502_13245_gb300 as rr
+    rr.build()
+    rr.load_library()
+    return rr
+
+
+def _graph(rng, n, R):
+    adj = rng.integers(0, n, size=(n, R)).astype(np.uint32)
+    adj[:, 0] = (np.arange(n) + 1) % n  # every point is reached
+    adj = np.sort(adj, axis=1)          # repeated entries of a row become padding (a row is a set)
+    adj[:, 1:][adj[:, 1:] == adj[:, :-1]] = 0xFFFFFFFF
+    return adj
+
+
+def _data(n, d, R, nq, seed, top=30):
+    rng = np.random.default_rng(seed)
+    X = rng.integers(0, top, size=(n, d), dtype=np.uint8)
+    return X, _graph(rng, n, R), rng.integers(0, top, size=(nq, d), dtype=np.uint8)
+
+
+def _radius(X, Q, share):
+    return float(np.percentile(((X[None].astype(np.int64) - Q[:20, None].astype(np.int64)) ** 2).sum(-1), share))
+
+
+def _same(res, o_ids, o_d):
+    for i in range(len(o_ids)):
+        ids, d = res.query(i)
+        assert np.array_equal(ids, o_ids[i]), i
+        assert np.array_equal(d.astype(np.int64), np.asarray(o_d[i]).astype(np.int64)), i
+
+
+@pytest.mark.parametrize("variant", ["doubling", "doubling_es", "doubling_warm"])
+def test_exact_counters_of_doubling_are_kept_by_the_warp_form(rr, variant):
+    """rr_query_stats.evals is what the GPU evaluated; the lookahead evaluates more than its rounds keep."""
+    X, adj, Q = _data(1500, 16, 20, 30, 1)
+    r = _radius(X, Q, 40)
+    gi, oi = rr.Index.from_arrays(X, adj, 0), oracle.Index(X, adj, 0)
+    o_ids, o_d, o_st = oracle.range_search(oi, Q, r, variant, beam=8, threads=os.cpu_count() or 4)
+    warp, cta = rr.rr_debug_count("round_warp"), rr.rr_debug_count("round_cta")
+    res = gi.range_search(Q, r, variant, beam=8, collect_stats=1)
+    rounds = int(res.stats["rounds"].max())
+    assert rounds > 2 and rr.rr_debug_count("round_cta") == cta and rr.rr_debug_count("round_warp") == warp + rounds
+    _same(res, o_ids, o_d)
+    for key in ("rounds", "distinct", "visits_beam"):
+        assert np.array_equal(res.stats[key], [s[key] for s in o_st])
+    assert np.all(res.stats["evals"] >= res.stats["distinct"])
+    _same(gi.range_search(Q, r, variant, beam=8), o_ids, o_d)
+    assert rr.rr_debug_count("round_cta") > cta
+    gi.close()
