@@ -455,7 +455,10 @@ rr_status rr_debug_set(const char *key, int64_t value);
 /* How often the library has taken a form of a phase, over all calls of the
  * process, for tests that a path is the one they mean (-1: unknown key):
  *   "beam_warp", "beam_cta"    beam phases by a warp or by a CTA per query
- *   "round_warp", "round_cta"  doubling rounds, likewise */
+ *   "round_warp", "round_cta"  doubling rounds, likewise
+ *   "greedy_cluster"           greedy phases by a cluster of CTAs per query
+ *   "greedy_handed"            queries these handed to the level kernels
+ *   "greedy_levels"            greedy phases by the level kernels from the start */
 int64_t rr_debug_count(const char *key);
 
 #ifdef __cplusplus

@@ -38,7 +38,7 @@ namespace rr {
 
 namespace {
 
-constexpr int kChunk = 128;          // items a warp reserves at a time
+constexpr int kChunk = kBfsChunk;    // items a warp reserves at a time
 constexpr int kCand = 32 + 128;      // first-seen ids a warp holds: a batch and a full row
 constexpr int kWarpBytes = 32 * 8 + kCand * 4;
 constexpr int kCtlBytes = 64;
@@ -325,6 +325,7 @@ __global__ void __launch_bounds__(kBfsThreads, 1) bfs_kernel(BfsArgs g) {
         if (chief) {
             g.slot_count[slot] = (int32_t)total;
             a.res_count[qi] = (int32_t)total;
+            atomicAdd(g.results, (unsigned long long)total);
             atomicAdd(g.done, 1);
             atomicMax(g.levels, (int32_t)L);
         }

@@ -31,6 +31,10 @@ bool bfs_shape(int64_t n, int64_t nq, BfsShape *s) {
 
 size_t bfs_front_bytes(const BfsShape &s) { return (size_t)s.clusters * 2 * s.fcap * 4; }
 
+int64_t bfs_list_slack(const BfsShape &s) {
+    return ((int64_t)s.clusters << s.cl_log2) * (s.threads / 32) * kBfsChunk;
+}
+
 rr_status launch_bfs(BfsArgs g, const BfsShape &s, cudaStream_t st, int dtype_code) {
     g.cl_log2 = s.cl_log2;
     g.bm_words = s.bm_words;

@@ -18,7 +18,7 @@ rr_status cuda_fail(cudaError_t e, const char *what);
 // all threads share: it is only ever raised, so that no launch finds it below what it asked for.
 rr_status allow_smem(const void *kernel, size_t bytes);
 // forms of the phases, counted for rr_debug_count
-enum Form { kFormBeamWarp, kFormBeamCta, kFormRoundWarp, kFormRoundCta, kForms };
+enum Form { kFormBeamWarp, kFormBeamCta, kFormRoundWarp, kFormRoundCta, kFormCluster, kFormHanded, kFormLevels, kForms };
 void note_form(Form f, int64_t k = 1);
 // failure-path hooks set by rr_debug_set: true if this device allocation is to fail;
 // the beam and doubling kernels' per-query iteration guard (default n + 1); the tries of a wait in the 8-bit
@@ -214,6 +214,7 @@ struct GreedyArgs {
 
 // Alg. 2 with a cluster of CTAs per query, bitmaps in shared memory (k_bfs.cuh).
 constexpr int kBfsThreads = 768;  // threads of a CTA
+constexpr int kBfsChunk = 128;    // entries of the item list that a warp reserves at a time
 struct BfsShape {
     int cl_log2, threads, clusters, bm_words;
     uint32_t fcap;             // entries of one frontier list (two a cluster)
@@ -225,6 +226,7 @@ struct BfsArgs {
     const int32_t *np2;        // queued queries
     int32_t *next, *done, *handed, *overflow, *levels;  // device counters, zero at the start
     unsigned long long *tail;  // item append cursor, zero at the start
+    unsigned long long *results;  // results of the finished queries, zero at the start
     uint64_t *item_key;
     int32_t *item_slot;        // -1: no item
     int64_t cap;
@@ -246,6 +248,8 @@ struct BfsArgs {
 // false: the index is too large for the bitmaps, the two-pass levels are the faster ones
 bool bfs_shape(int64_t n, int64_t nq, BfsShape *s);
 size_t bfs_front_bytes(const BfsShape &s);
+// entries of the item list without an item, at most (a warp reserves whole chunks)
+int64_t bfs_list_slack(const BfsShape &s);
 rr_status launch_bfs(BfsArgs g, const BfsShape &s, cudaStream_t st, int dtype_code);
 
 rr_status launch_greedy_init(const GreedyArgs &g, cudaStream_t s, int dtype_code);

@@ -18,7 +18,7 @@ size_t ru(size_t x) { return (x + 255) & ~size_t(255); }
 
 // device counter words (zeroed before the beam phase): queued queries, status, work queues and the item cursor
 enum { kCtrP2 = 0, kCtrError = 1, kCtrNextQ = 2, kCtrBfsNext = 3, kCtrBfsDone = 4, kCtrHand = 5, kCtrOverflow = 6,
-       kCtrLevels = 7, kCtrTail = 8, kCtrCand = 10, kCtrPend = 12, kCtrWords = 16 };
+       kCtrLevels = 7, kCtrTail = 8, kCtrCand = 10, kCtrPend = 12, kCtrResults = 14, kCtrWords = 16 };
 
 struct Search {
     rr_index *ix;
@@ -286,14 +286,18 @@ struct GreedyOut {
     int64_t nitems = 0;
 };
 
-// Queries that the cluster kernel handed to the two-pass levels: their pending items, bitmaps, and the items so far.
+// Queries that the cluster kernel handed to the two-pass levels: their pending items, bitmaps, the item list's end and
+// the results in it so far (the rest of its entries are empty).
 struct HandOver {
     const uint64_t *key;
     const int32_t *slot;
     int64_t count;
     uint32_t *bits;
-    int64_t tail;
+    int64_t tail, results;
 };
+
+// max_results_total bounds the results of the phase; the first beams are always kept
+int64_t result_cap(const Search &S, int64_t np2) { return std::max<int64_t>(S.P.max_results_total, np2 * S.a.beam); }
 
 // Alg. 2 level by level (see k_greedy.cu) for the np2 queued queries, or from where the cluster kernel left the
 // handed-over ones.  *capped: an item found no room within max_results_total.
@@ -322,7 +326,7 @@ rr_status run_greedy(Search &S, int32_t np2, const HandOver *ho, GreedyOut &go, 
         g.seen = (uint32_t *)ix->phase2.p;
         RR_CUDA(cudaMemsetAsync(g.seen, 0, (size_t)np2 * words * 4, S.st));
     }
-    const int64_t cap_limit = std::max<int64_t>(S.P.max_results_total, init);
+    const int64_t cap_limit = result_cap(S, np2) + (ho ? ho->tail - ho->results : 0);  // empty entries do not count
     const int64_t want = std::min<int64_t>(cap_limit, std::max<int64_t>(ho ? init : init * 8, (int64_t)1 << 20));
     if ((s = grow(ix->item_key, (size_t)want * 8, ho ? (size_t)init * 8 : 0, S.st)) != RR_OK) return s;
     if ((s = grow(ix->item_slot, (size_t)want * 4, ho ? (size_t)init * 4 : 0, S.st)) != RR_OK) return s;
@@ -343,6 +347,7 @@ rr_status run_greedy(Search &S, int32_t np2, const HandOver *ho, GreedyOut &go, 
     int64_t begin = 0, end = ho ? ho->count : init, tail = init, levels = 0;
     bool pending = ho != nullptr;
     *capped = false;
+    if (!ho) note_form(kFormLevels);
     while (begin < end) {
         const int64_t need = tail + (end - begin) * (int64_t)ix->R;
         if (need > g.cap && g.cap < cap_limit) {
@@ -398,14 +403,15 @@ constexpr int kHandSlots = 24, kHandCap = 32;
 
 // Alg. 2 for the queued queries, a cluster of CTAs each (k_bfs.cuh), and the scan of the final counts; their number
 // is read back only after both.  Queries handed over by the kernel are finished by the two-pass levels.  If the
-// items hit their list's end or max_results_total, all queries are redone by the two-pass levels, which grow the
-// list and cut results at the cap.
+// items hit their list's end or the results max_results_total, all queries are redone by the two-pass levels, which
+// grow the list and cut results at the cap.
 rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go) {
     rr_index *ix = S.ix;
     const SearchArgs &a = S.a;
     const int64_t words = (ix->n + 31) / 32;
     rr_status s;
-    const int64_t want = std::min<int64_t>(S.P.max_results_total, (int64_t)1 << 22);
+    const int64_t slack = bfs_list_slack(shape);
+    const int64_t want = std::min<int64_t>(result_cap(S, S.nq), (int64_t)1 << 22) + slack;
     if ((s = grow(ix->item_key, (size_t)want * 8, 0, S.st)) != RR_OK) return s;
     if ((s = grow(ix->item_slot, (size_t)want * 4, 0, S.st)) != RR_OK) return s;
     if ((s = grow(ix->front, bfs_front_bytes(shape), 0, S.st)) != RR_OK) return s;
@@ -426,7 +432,8 @@ rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go)
     g.tail = S.tail;
     g.item_key = (uint64_t *)ix->item_key.p;
     g.item_slot = (int32_t *)ix->item_slot.p;
-    g.cap = std::min<int64_t>(S.P.max_results_total, (int64_t)std::min(ix->item_key.bytes / 8, ix->item_slot.bytes / 4));
+    g.results = (unsigned long long *)(S.counters + kCtrResults);
+    g.cap = (int64_t)std::min(ix->item_key.bytes / 8, ix->item_slot.bytes / 4);
     g.slot_count = S.slot_count;
     g.front = (uint32_t *)ix->front.p;
     g.bail_total = kHandTotal;
@@ -439,17 +446,21 @@ rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go)
     g.hand_words = words;
     g.pend_key = (uint64_t *)((uint8_t *)ix->hand.p + off_pk);
     g.pend_slot = (int32_t *)((uint8_t *)ix->hand.p + off_ps);
+    note_form(kFormCluster);
     if ((s = launch_bfs(g, shape, S.st, ix->dtype)) != RR_OK) return s;
     if (S.prof_ev) RR_CUDA(cudaEventRecord(S.prof_ev, S.st));
     if ((s = scan_counts(S)) != RR_OK) return s;
     *np2 = S.hc[kCtrP2];
     S.phase2_steps = S.hc[kCtrLevels];
-    unsigned long long tail;
+    unsigned long long tail, results;
     memcpy(&tail, S.hc + kCtrTail, 8);
-    bool capped = S.hc[kCtrOverflow] != 0 || (int64_t)tail > g.cap;
+    memcpy(&results, S.hc + kCtrResults, 8);
+    bool capped = S.hc[kCtrOverflow] != 0 || (int64_t)tail > g.cap || (int64_t)results > result_cap(S, *np2);
     go.nitems = (int64_t)tail;
     if (!capped && S.hc[kCtrHand] > 0) {
-        const HandOver ho{g.pend_key, g.pend_slot, (int64_t)(uint32_t)S.hc[kCtrPend], g.hand_bits, (int64_t)tail};
+        const HandOver ho{g.pend_key, g.pend_slot, (int64_t)(uint32_t)S.hc[kCtrPend], g.hand_bits, (int64_t)tail,
+                          (int64_t)results};
+        note_form(kFormHanded, S.hc[kCtrHand]);
         if ((s = run_greedy(S, *np2, &ho, go, &capped)) != RR_OK) return s;
     }
     if (capped && (s = run_greedy(S, *np2, nullptr, go, &capped)) != RR_OK) return s;

@@ -64,3 +64,26 @@ def test_exact_counters_of_doubling_are_kept_by_the_warp_form(rr, variant):
     _same(gi.range_search(Q, r, variant, beam=8), o_ids, o_d)
     assert rr.rr_debug_count("round_cta") > cta
     gi.close()
+
+
+def test_cap_counts_results_not_list_entries(rr):
+    """The cluster expansion's warps reserve the item list in chunks and leave most of a small batch's empty; only
+    results count against max_results_total.  At the exact number of results nothing is cut and nothing is redone;
+    one less cuts."""
+    X, adj, Q = _data(3000, 16, 20, 200, 2)
+    r = _radius(X, Q, 10)
+    gi, oi = rr.Index.from_arrays(X, adj, 0), oracle.Index(X, adj, 0)
+    beam = 8
+    o_ids, o_d, _ = oracle.range_search(oi, Q, r, "greedy", beam=beam, threads=os.cpu_count() or 4)
+    counts = np.array([len(x) for x in o_ids])
+    full = int(counts[counts >= beam].sum())
+    assert full > beam * (counts >= beam).sum()
+    for cap in (full + 1, full):
+        cluster, levels = rr.rr_debug_count("greedy_cluster"), rr.rr_debug_count("greedy_levels")
+        res = gi.range_search(Q, r, "greedy", beam=beam, max_results_total=cap)
+        assert res.status == rr.RR_OK and not np.any(res.flags & rr.RR_FLAG_TRUNCATED)
+        assert rr.rr_debug_count("greedy_cluster") == cluster + 1 and rr.rr_debug_count("greedy_levels") == levels
+        _same(res, o_ids, o_d)
+    res = gi.range_search(Q, r, "greedy", beam=beam, max_results_total=full - 1)
+    assert res.status == rr.RR_EOVERFLOW and len(res.ids) == counts.sum() - 1
+    gi.close()
