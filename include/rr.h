@@ -457,6 +457,7 @@ rr_status rr_debug_set(const char *key, int64_t value);
  *   "beam_warp", "beam_cta"    beam phases by a warp or by a CTA per query
  *   "round_warp", "round_cta"  doubling rounds, likewise
  *   "greedy_cluster"           greedy phases by a cluster of CTAs per query
+ *   "greedy_again"             of these, run a second time with a longer list
  *   "greedy_handed"            queries these handed to the level kernels
  *   "greedy_levels"            greedy phases by the level kernels from the start */
 int64_t rr_debug_count(const char *key);

@@ -187,9 +187,7 @@ __global__ void __launch_bounds__(kBfsThreads, 1) bfs_kernel(BfsArgs g) {
                 if (at < g.cap) {
                     g.item_key[at] = k;
                     g.item_slot[at] = slot;
-                } else {
-                    *g.overflow = 1;  // the host redoes the phase with a larger list
-                }
+                }  // else the cursor says how long a list the host has to bring
                 if (fc && f0 + p < g.fcap) f[f0 + p] = key_id(k);
             }
             if (cnt > room) {

@@ -18,7 +18,7 @@ rr_status cuda_fail(cudaError_t e, const char *what);
 // all threads share: it is only ever raised, so that no launch finds it below what it asked for.
 rr_status allow_smem(const void *kernel, size_t bytes);
 // forms of the phases, counted for rr_debug_count
-enum Form { kFormBeamWarp, kFormBeamCta, kFormRoundWarp, kFormRoundCta, kFormCluster, kFormHanded, kFormLevels, kForms };
+enum Form { kFormBeamWarp, kFormBeamCta, kFormRoundWarp, kFormRoundCta, kFormCluster, kFormClusterAgain, kFormHanded, kFormLevels, kForms };
 void note_form(Form f, int64_t k = 1);
 // failure-path hooks set by rr_debug_set: true if this device allocation is to fail;
 // the beam and doubling kernels' per-query iteration guard (default n + 1); the tries of a wait in the 8-bit
@@ -224,7 +224,8 @@ struct BfsArgs {
     SearchArgs s;
     const int32_t *qlist;      // slot -> query
     const int32_t *np2;        // queued queries
-    int32_t *next, *done, *handed, *overflow, *levels;  // device counters, zero at the start
+    int32_t *next, *done, *handed, *overflow, *levels;  // device counters, zero at the start (overflow: a frontier or
+                                                        // a handed-over query found no room)
     unsigned long long *tail;  // item append cursor, zero at the start
     unsigned long long *results;  // results of the finished queries, zero at the start
     uint64_t *item_key;

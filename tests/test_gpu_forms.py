@@ -87,3 +87,39 @@ def test_cap_counts_results_not_list_entries(rr):
     res = gi.range_search(Q, r, "greedy", beam=beam, max_results_total=full - 1)
     assert res.status == rr.RR_EOVERFLOW and len(res.ids) == counts.sum() - 1
     gi.close()
+
+
+def _all_in_range(n, m, R, nq, seed):
+    """m of n points joined by a random graph, a radius that holds all of them: every query's results are all m."""
+    rng = np.random.default_rng(seed)
+    live = np.sort(rng.choice(n, m, replace=False))
+    live[0], live[-1] = 0, n - 1
+    adj = np.full((n, R), 0xFFFFFFFF, np.uint32)
+    row = live[rng.integers(0, m, size=(m, R))].astype(np.uint32)
+    row[:, 0] = np.roll(live, -1)
+    row = np.sort(row, axis=1)
+    row[:, 1:][row[:, 1:] == row[:, :-1]] = 0xFFFFFFFF
+    adj[live] = row
+    X = np.zeros((n, 8), np.uint8)
+    X[live] = rng.integers(0, 200, size=(m, 8))
+    return X, adj, live, rng.integers(0, 200, size=(nq, 8), dtype=np.uint8)
+
+
+def _check_all(res, X, live, Q):
+    for i in range(len(Q)):
+        d2 = ((X[live].astype(np.int64) - Q[i].astype(np.int64)) ** 2).sum(-1)
+        o = np.lexsort((live, d2))
+        ids, d = res.query(i)
+        assert np.array_equal(ids, live[o]) and np.array_equal(d.astype(np.int64), d2[o]), i
+
+
+def test_short_item_list_is_grown_and_the_clusters_run_again(rr):
+    """5 M results on a fresh index: the first list is too short; the second run fits, and the next call at once."""
+    X, adj, live, Q = _all_in_range(60_000, 50_000, 24, 100, 3)
+    gi = rr.Index.from_arrays(X, adj, 0)
+    for again in (1, 0):
+        before = [rr.rr_debug_count("greedy_" + k) for k in ("again", "levels")]
+        res = gi.range_search(Q, 1e9, "greedy", beam=16)
+        assert [rr.rr_debug_count("greedy_" + k) for k in ("again", "levels")] == [before[0] + again, before[1]]
+        _check_all(res, X, live, Q)
+    gi.close()
