@@ -42,10 +42,13 @@ constexpr int kChunk = kBfsChunk;    // items a warp reserves at a time
 constexpr int kCand = 32 + 128;      // first-seen ids a warp holds: a batch and a full row
 constexpr int kWarpBytes = 32 * 8 + kCand * 4;
 constexpr int kCtlBytes = 64;
+constexpr int kHandOver = 1, kStop = 2;
+constexpr uint32_t kStopFront = 1024;  // smaller frontiers do not ask for the cursor: the next query does
 
 struct Ctl {                         // the copies of the cluster's first CTA are used
     int32_t slot;
-    int32_t bail[2];                 // by level parity: written during a level, read after the barrier that ends it
+    int32_t bail[2];                 // kHandOver or kStop, by level parity: written during a level, read after the
+                                     // barrier that ends it
     int32_t hand;                    // hand-over: the query's bitmap in global memory, or -1
     uint32_t pend;                   // and its place in the list of pending items
     uint32_t cnt[3];                 // frontier sizes of three consecutive levels
@@ -141,13 +144,20 @@ __global__ void __launch_bounds__(kBfsThreads, 1) bfs_kernel(BfsArgs g) {
     uint32_t *fr = g.front + (size_t)(blockIdx.x >> T.log2) * 2 * g.fcap;
     const bool chief = T.rank == 0 && threadIdx.x == 0;
     const int32_t np2 = *g.np2;
+    // the list's cursor shows more results than the caller's cap (first beams are always kept)
+    auto beyond_cap = [&]() {
+        return *(volatile unsigned long long *)g.tail >
+               (unsigned long long)(max(g.max_results, (int64_t)np2 * b) + g.slack);
+    };
     // this warp's chunk of the item list
     int64_t cbase = 0;
     int cfill = kChunk;
 
     for (;;) {
         if (chief) {
-            T.ctl->slot = atomicAdd(g.next, 1);
+            const bool full = beyond_cap();
+            if (full) *g.overflow = 1;
+            T.ctl->slot = full ? np2 : atomicAdd(g.next, 1);
             T.ctl->bail[0] = T.ctl->bail[1] = 0;
             T.ctl->cnt[0] = (uint32_t)b;
             T.ctl->cnt[1] = 0;
@@ -210,7 +220,7 @@ __global__ void __launch_bounds__(kBfsThreads, 1) bfs_kernel(BfsArgs g) {
         }
         T.sync();
         uint32_t total = (uint32_t)b, L = 0;
-        bool bail = false;
+        int32_t bail = 0;
         for (;; L++) {
             const uint32_t F = L == 0 ? (uint32_t)b : T.get(&T.ctl->cnt[L % 3]);
             if (L > 0) {
@@ -219,7 +229,7 @@ __global__ void __launch_bounds__(kBfsThreads, 1) bfs_kernel(BfsArgs g) {
                     if (chief) *g.overflow = 1;
                     break;
                 }
-                bail = T.get(&T.ctl->bail[L & 1]) != 0;
+                bail = (int32_t)T.get(&T.ctl->bail[L & 1]);
                 if (F == 0 || bail) break;
             }
             const uint32_t *fin = fr + (size_t)(L & 1) * g.fcap;
@@ -228,7 +238,11 @@ __global__ void __launch_bounds__(kBfsThreads, 1) bfs_kernel(BfsArgs g) {
             if (chief) {
                 T.ctl->cnt[(L + 2) % 3] = 0;
                 if (total >= g.bail_total && F >= g.bail_front && np2 - *(volatile int32_t *)g.done <= g.bail_slots)
-                    T.ctl->bail[(L + 1) & 1] = 1;
+                    T.ctl->bail[(L + 1) & 1] = kHandOver;
+                if (F >= kStopFront && beyond_cap()) {
+                    T.ctl->bail[(L + 1) & 1] = kStop;
+                    *g.overflow = 1;
+                }
             }
             // a small frontier: 2^sp warps share an item, each taking every 2^sp-th entry of its row, so that the
             // evaluations (several gather round trips a warp) spread over the team
@@ -292,7 +306,7 @@ __global__ void __launch_bounds__(kBfsThreads, 1) bfs_kernel(BfsArgs g) {
             if (nc > 0) evaluate(nc);
             T.sync();
         }
-        if (bail) {
+        if (bail == kHandOver) {
             // hand over: the next frontier (its points are results already) and the bitmap
             const uint32_t F = T.get(&T.ctl->cnt[L % 3]);
             if (chief) {

@@ -225,12 +225,13 @@ struct BfsArgs {
     const int32_t *qlist;      // slot -> query
     const int32_t *np2;        // queued queries
     int32_t *next, *done, *handed, *overflow, *levels;  // device counters, zero at the start (overflow: a frontier or
-                                                        // a handed-over query found no room)
+                                                        // a handed-over query found no room, or max_results)
     unsigned long long *tail;  // item append cursor, zero at the start
     unsigned long long *results;  // results of the finished queries, zero at the start
     uint64_t *item_key;
     int32_t *item_slot;        // -1: no item
     int64_t cap;
+    int64_t max_results, slack;  // the clusters stop (overflow) once the list shows more results than the caller's cap
     int32_t *slot_count;       // results per slot (so far, for a query handed over)
     uint32_t *front;           // clusters x 2 x fcap
     uint32_t fcap;

@@ -434,6 +434,8 @@ rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go)
     g.pend_count = (uint32_t *)(S.counters + kCtrPend);
     g.tail = S.tail;
     g.results = (unsigned long long *)(S.counters + kCtrResults);
+    g.max_results = S.P.max_results_total;
+    g.slack = slack;
     g.slot_count = S.slot_count;
     g.front = (uint32_t *)ix->front.p;
     g.bail_total = kHandTotal;
@@ -459,7 +461,7 @@ rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go)
         memcpy(&tail, S.hc + kCtrTail, 8);
         memcpy(&results, S.hc + kCtrResults, 8);
         *np2 = S.hc[kCtrP2];
-        capped = S.hc[kCtrOverflow] != 0 || results > result_cap(S, *np2);
+        capped = S.hc[kCtrOverflow] != 0 || results > result_cap(S, *np2);  // a run that stopped: overflow
         if (capped || tail <= g.cap) break;
         want = results + slack;
         if ((s = grow(ix->item_key, (size_t)want * 8, 0, S.st)) != RR_OK) return s;

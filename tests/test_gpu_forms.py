@@ -123,3 +123,27 @@ def test_short_item_list_is_grown_and_the_clusters_run_again(rr):
         assert [rr.rr_debug_count("greedy_" + k) for k in ("again", "levels")] == [before[0] + again, before[1]]
         _check_all(res, X, live, Q)
     gi.close()
+
+
+def test_a_capped_call_does_not_expand_everything_first(rr):
+    """Results beyond max_results_total are cut by the level kernels; the clusters stop once the cap is exceeded."""
+    X, adj, live, Q = _all_in_range(60_000, 50_000, 24, 100, 4)
+    gi = rr.Index.from_arrays(X, adj, 0)
+
+    def phase2_ms(**kw):
+        best = 1e9
+        for _ in range(5):
+            res = gi.range_search(Q, 1e9, "greedy", beam=16, profile=1, **kw)
+            best = min(best, rr.rr_last_profile(gi.h).phase2_ms)
+        return best, res
+
+    full, res = phase2_ms()
+    _check_all(res, X, live, Q)
+    levels = rr.rr_debug_count("greedy_levels")
+    capped, res = phase2_ms(max_results_total=20_000)
+    assert rr.rr_debug_count("greedy_levels") == levels + 5
+    assert res.status == rr.RR_EOVERFLOW and len(res.ids) == 20_000
+    assert np.all((res.flags & rr.RR_FLAG_TRUNCATED) != 0)
+    assert capped < full, (capped, full)  # both forms one after the other took longer than the full expansion
+    _check_all(gi.range_search(Q, 1e9, "greedy", beam=16), X, live, Q)
+    gi.close()
