@@ -22,7 +22,8 @@
 //
 // The last few large queries, once the rest of the chip has run dry, are handed
 // to the two-pass levels (bitmap and frontier are copied out): a CTA does ~3
-// probes per clock, the flat passes ~86 over the chip.
+// probes per clock, the flat passes ~86 over the chip.  So is a query whose
+// frontier outgrows its list.
 //
 // Measured (GB300, greedy phase): 836 queries, 5.6 M results, 2*10^6 x 256 u8
 // 2.62 -> 1.32 ms; 1,163 queries, 36.0 M results 18.3 -> 9.2 ms; 265 queries,
@@ -43,7 +44,6 @@ constexpr int kCand = 32 + 128;      // first-seen ids a warp holds: a batch and
 constexpr int kWarpBytes = 32 * 8 + kCand * 4;
 constexpr int kCtlBytes = 64;
 constexpr int kHandOver = 1, kStop = 2;
-constexpr uint32_t kStopFront = 1024;  // smaller frontiers do not ask for the cursor: the next query does
 
 struct Ctl {                         // the copies of the cluster's first CTA are used
     int32_t slot;
@@ -144,10 +144,11 @@ __global__ void __launch_bounds__(kBfsThreads, 1) bfs_kernel(BfsArgs g) {
     uint32_t *fr = g.front + (size_t)(blockIdx.x >> T.log2) * 2 * g.fcap;
     const bool chief = T.rank == 0 && threadIdx.x == 0;
     const int32_t np2 = *g.np2;
-    // the list's cursor shows more results than the caller's cap (first beams are always kept)
-    auto beyond_cap = [&]() {
-        return *(volatile unsigned long long *)g.tail >
-               (unsigned long long)(max(g.max_results, (int64_t)np2 * b) + g.slack);
+    // the caller's cap on the results (first beams are always kept), and the end of a run that will be redone
+    auto cap = [&]() { return (unsigned long long)max(g.max_results, (int64_t)np2 * b); };
+    auto give_up = [&]() {
+        *g.overflow = 1;
+        atomicMax(g.next, np2);  // no more queries
     };
     // this warp's chunk of the item list
     int64_t cbase = 0;
@@ -155,9 +156,13 @@ __global__ void __launch_bounds__(kBfsThreads, 1) bfs_kernel(BfsArgs g) {
 
     for (;;) {
         if (chief) {
-            const bool full = beyond_cap();
-            if (full) *g.overflow = 1;
-            T.ctl->slot = full ? np2 : atomicAdd(g.next, 1);
+            const unsigned long long found = *(volatile unsigned long long *)g.results;  // both in flight together
+            const int32_t next = atomicAdd(g.next, 1);
+            T.ctl->slot = next;
+            if (found > cap()) {
+                give_up();
+                T.ctl->slot = np2;
+            }
             T.ctl->bail[0] = T.ctl->bail[1] = 0;
             T.ctl->cnt[0] = (uint32_t)b;
             T.ctl->cnt[1] = 0;
@@ -225,11 +230,8 @@ __global__ void __launch_bounds__(kBfsThreads, 1) bfs_kernel(BfsArgs g) {
             const uint32_t F = L == 0 ? (uint32_t)b : T.get(&T.ctl->cnt[L % 3]);
             if (L > 0) {
                 total += F;
-                if (F > g.fcap) {
-                    if (chief) *g.overflow = 1;
-                    break;
-                }
                 bail = (int32_t)T.get(&T.ctl->bail[L & 1]);
+                if (F > g.fcap && !bail) bail = kHandOver;
                 if (F == 0 || bail) break;
             }
             const uint32_t *fin = fr + (size_t)(L & 1) * g.fcap;
@@ -239,9 +241,9 @@ __global__ void __launch_bounds__(kBfsThreads, 1) bfs_kernel(BfsArgs g) {
                 T.ctl->cnt[(L + 2) % 3] = 0;
                 if (total >= g.bail_total && F >= g.bail_front && np2 - *(volatile int32_t *)g.done <= g.bail_slots)
                     T.ctl->bail[(L + 1) & 1] = kHandOver;
-                if (F >= kStopFront && beyond_cap()) {
+                if (F >= g.bail_front && *(volatile unsigned long long *)g.tail > cap() + g.slack) {
                     T.ctl->bail[(L + 1) & 1] = kStop;
-                    *g.overflow = 1;
+                    give_up();
                 }
             }
             // a small frontier: 2^sp warps share an item, each taking every 2^sp-th entry of its row, so that the
@@ -307,23 +309,26 @@ __global__ void __launch_bounds__(kBfsThreads, 1) bfs_kernel(BfsArgs g) {
             T.sync();
         }
         if (bail == kHandOver) {
-            // hand over: the next frontier (its points are results already) and the bitmap
+            // hand over: the bitmap, and the next frontier (its points are results already).  One that has outgrown
+            // its list is marked instead; the host takes all the query's results for it.
             const uint32_t F = T.get(&T.ctl->cnt[L % 3]);
+            const uint32_t f = F > g.fcap ? 0u : F;
             if (chief) {
-                const int h = atomicAdd(g.handed, 1);
-                const uint32_t p = atomicAdd(g.pend_count, F);
-                const bool fits = h < g.hand_cap && p + F <= g.pend_cap && p + F >= p;
-                if (!fits) *g.overflow = 1;
-                T.ctl->hand = fits ? h : -1;
+                const unsigned long long w = atomicAdd(g.hand_pend, (1ull << 32) + f);
+                const uint32_t h = (uint32_t)(w >> 32), p = (uint32_t)w;
+                const bool fits = h < (uint32_t)g.hand_cap && p + f <= g.pend_cap && p + f >= p;
+                if (!fits) give_up();
+                T.ctl->hand = fits ? (int32_t)h : -1;
                 T.ctl->pend = p;
-                if (fits) g.hand_of[slot] = h;
+                if (fits) g.hand_of[slot] = (int32_t)h;
+                if (fits && F > g.fcap) g.outgrown[h] = slot + 1;
             }
             T.sync();
             const int32_t h = (int32_t)T.get(&T.ctl->hand);
             if (h >= 0) {
                 const uint32_t p = T.get(&T.ctl->pend);
                 const uint32_t *fin = fr + (size_t)(L & 1) * g.fcap;
-                for (uint32_t i = T.rank * blockDim.x + threadIdx.x; i < F; i += blockDim.x << T.log2) {
+                for (uint32_t i = T.rank * blockDim.x + threadIdx.x; i < f; i += blockDim.x << T.log2) {
                     g.pend_key[p + i] = make_key(0, __ldcg(fin + i));
                     g.pend_slot[p + i] = slot;
                 }

@@ -480,6 +480,21 @@ __global__ void count_items_kernel(const int32_t *item_slot, int64_t n, int32_t 
     }
 }
 
+// the items of the listed slots (queries whose frontier outgrew its list: rare), in any order
+__global__ void gather_slots_kernel(const uint64_t *item_key, const int32_t *item_slot, int64_t n, SlotList list,
+                                    uint64_t *key, int32_t *slot, int64_t cap, unsigned long long *at) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t s = item_slot[t];
+        bool in = false;
+        for (int i = 0; i < list.n; i++) in |= s >= 0 && list.slot1[i] == s + 1;
+        if (!in) continue;
+        const unsigned long long p = atomicAdd(at, 1ull);
+        if (p >= (unsigned long long)cap) continue;
+        key[p] = item_key[t];
+        slot[p] = s;
+    }
+}
+
 __global__ void set_counts_kernel(int32_t *res_count, uint8_t *flags, const int32_t *qlist, const int32_t *slot_count,
                                   const int32_t *slot_trunc, int32_t n) {
     for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
@@ -534,6 +549,16 @@ rr_status launch_count_items(const int32_t *item_slot, int64_t n, int32_t *slot_
     if (n <= 0) return RR_OK;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 16));
     count_items_kernel<<<(unsigned)blocks, 256, 0, st>>>(item_slot, n, slot_count);
+    RR_CUDA(cudaGetLastError());
+    note_launch();
+    return RR_OK;
+}
+
+rr_status launch_gather_slots(const uint64_t *item_key, const int32_t *item_slot, int64_t n, const SlotList &list,
+                              uint64_t *key, int32_t *slot, int64_t cap, unsigned long long *at, cudaStream_t st) {
+    if (n <= 0 || list.n <= 0) return RR_OK;
+    const int64_t blocks = std::min<int64_t>((n + 255) / 256, 152 * 16);
+    gather_slots_kernel<<<(unsigned)blocks, 256, 0, st>>>(item_key, item_slot, n, list, key, slot, cap, at);
     RR_CUDA(cudaGetLastError());
     note_launch();
     return RR_OK;

@@ -88,6 +88,7 @@ struct rr_index {
     rr::Grow cand;          // greedy candidate list of a level chunk (8-bit indexes)
     rr::Grow front;         // greedy frontier lists
     rr::Grow hand;          // greedy queries handed from the cluster kernel to the two-pass levels
+    rr::Grow outgrown;      // their pending items, when a frontier outgrew its list
     rr::Grow dbl_seen;      // warm-restart doubling: per-query bitmaps of every id evaluated
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // profile: start, beam, phase2, end
     rr_profile prof = {};
@@ -214,6 +215,7 @@ struct GreedyArgs {
 
 // Alg. 2 with a cluster of CTAs per query, bitmaps in shared memory (k_bfs.cuh).
 constexpr int kBfsThreads = 768;  // threads of a CTA
+constexpr int kBfsHandCap = 32;   // queries handed over in a call, at most
 constexpr int kBfsChunk = 128;    // entries of the item list that a warp reserves at a time
 struct BfsShape {
     int cl_log2, threads, clusters, bm_words;
@@ -224,14 +226,15 @@ struct BfsArgs {
     SearchArgs s;
     const int32_t *qlist;      // slot -> query
     const int32_t *np2;        // queued queries
-    int32_t *next, *done, *handed, *overflow, *levels;  // device counters, zero at the start (overflow: a frontier or
+    int32_t *next, *done, *overflow, *levels;  // device counters, zero at the start (overflow: a frontier or
                                                         // a handed-over query found no room, or max_results)
     unsigned long long *tail;  // item append cursor, zero at the start
     unsigned long long *results;  // results of the finished queries, zero at the start
     uint64_t *item_key;
     int32_t *item_slot;        // -1: no item
     int64_t cap;
-    int64_t max_results, slack;  // the clusters stop (overflow) once the list shows more results than the caller's cap
+    int64_t max_results, slack;  // the clusters stop (overflow) once the results, or the list's cursor by more than
+                                 // slack, exceed the caller's cap
     int32_t *slot_count;       // results per slot (so far, for a query handed over)
     uint32_t *front;           // clusters x 2 x fcap
     uint32_t fcap;
@@ -240,7 +243,8 @@ struct BfsArgs {
     int32_t bail_slots;               // when at most bail_slots queries are unfinished
     int32_t hand_cap;          // room for handed-over bitmaps (hand_words each) and pending items
     uint32_t pend_cap;
-    uint32_t *pend_count;      // zero at the start
+    unsigned long long *hand_pend;  // queries handed over (high word) and pending items (low word), zero at the start
+    int32_t *outgrown;         // by bitmap: slot + 1 of a query whose frontier outgrew its list, zero at the start
     int32_t *hand_of;
     uint32_t *hand_bits;
     int64_t hand_words;
@@ -253,6 +257,13 @@ size_t bfs_front_bytes(const BfsShape &s);
 // entries of the item list without an item, at most (a warp reserves whole chunks)
 int64_t bfs_list_slack(const BfsShape &s);
 rr_status launch_bfs(BfsArgs g, const BfsShape &s, cudaStream_t st, int dtype_code);
+
+// appends the items of the slots in list (entries 0: none) to key / slot from *at on
+struct SlotList {
+    int32_t n, slot1[kBfsHandCap];  // slot + 1
+};
+rr_status launch_gather_slots(const uint64_t *item_key, const int32_t *item_slot, int64_t n, const SlotList &list,
+                              uint64_t *key, int32_t *slot, int64_t cap, unsigned long long *at, cudaStream_t s);
 
 rr_status launch_greedy_init(const GreedyArgs &g, cudaStream_t s, int dtype_code);
 rr_status launch_greedy_level(const GreedyArgs &g, cudaStream_t s, int dtype_code);

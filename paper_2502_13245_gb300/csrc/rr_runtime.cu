@@ -346,6 +346,7 @@ rr_status rr_free_index(rr_index *ix) {
     grow_free(ix->dbl_seen);
     grow_free(ix->front);
     grow_free(ix->hand);
+    grow_free(ix->outgrown);
     for (int k = 0; k < 4; k++)
         if (ix->ev[k]) cudaEventDestroy(ix->ev[k]);
     if (ix->lp_bf16) cudaFree(ix->lp_bf16);
@@ -363,7 +364,7 @@ rr_status rr_index_info_get(const rr_index *ix, rr_index_info *info) {
     info->device = ix->device;
     info->scratch_bytes = (int64_t)ix->arena.cap + (int64_t)ix->phase2.bytes + (int64_t)ix->item_key.bytes +
                           (int64_t)ix->item_slot.bytes + (int64_t)ix->outbuf.bytes + (int64_t)ix->dbl_s[0].bytes +
-                          (int64_t)ix->dbl_s[1].bytes + (int64_t)ix->dbl_tmp.bytes + (int64_t)ix->cand.bytes + (int64_t)ix->dbl_seen.bytes + (int64_t)ix->front.bytes + (int64_t)ix->hand.bytes +
+                          (int64_t)ix->dbl_s[1].bytes + (int64_t)ix->dbl_tmp.bytes + (int64_t)ix->cand.bytes + (int64_t)ix->dbl_seen.bytes + (int64_t)ix->front.bytes + (int64_t)ix->hand.bytes + (int64_t)ix->outgrown.bytes +
                           (int64_t)ix->pinned.cap;
     info->order = ix->order;
     info->reserved = 0;

@@ -17,9 +17,11 @@ namespace {
 size_t ru(size_t x) { return (x + 255) & ~size_t(255); }
 
 // device counter words (zeroed before the beam phase): queued queries, status, work queues and the item cursor
-enum { kCtrP2 = 0, kCtrError = 1, kCtrNextQ = 2, kCtrBfsNext = 3, kCtrBfsDone = 4, kCtrHand = 5, kCtrOverflow = 6,
-       kCtrLevels = 7, kCtrTail = 8, kCtrCand = 10, kCtrPend = 12, kCtrResults = 14, kCtrWords = 16 };
+enum { kCtrP2 = 0, kCtrError = 1, kCtrNextQ = 2, kCtrBfsNext = 3, kCtrBfsDone = 4, kCtrOverflow = 6,
+       kCtrLevels = 7, kCtrTail = 8, kCtrCand = 10, kCtrPend = 12, kCtrResults = 14, kCtrOutgrown = 16,
+       kCtrWords = kCtrOutgrown + kBfsHandCap };
 // those of the cluster expansion: from kCtrBfsNext on
+static_assert(kCtrWords * 4 <= 256, "the counter block");
 
 struct Search {
     rr_index *ix;
@@ -400,14 +402,40 @@ rr_status run_greedy(Search &S, int32_t np2, const HandOver *ho, GreedyOut &go, 
 // When the cluster kernel hands a query over: a CTA expands ~3 probes per clock, the two-pass levels ~86 over the
 // chip but at ~30 us of launches and host round trip a level, so it pays for large frontiers of the last queries.
 constexpr uint32_t kHandTotal = 8192, kHandFront = 4096, kPendCap = 1u << 22;
-constexpr int kHandSlots = 24, kHandCap = 32;
+constexpr int kHandSlots = 24, kHandCap = kBfsHandCap;
+
+// Queries whose frontier outgrew its list: all their results go to the pending items.  Those expanded before find
+// every bit set, so the levels go on from the others.
+rr_status take_outgrown(Search &S, const BfsArgs &g, const SlotList &out, HandOver &ho) {
+    rr_index *ix = S.ix;
+    rr_status s;
+    int64_t most = ho.count;
+    std::vector<int32_t> count((size_t)out.n);
+    for (int i = 0; i < out.n; i++)
+        RR_CUDA(cudaMemcpyAsync(&count[(size_t)i], S.slot_count + out.slot1[i] - 1, 4, cudaMemcpyDeviceToHost, S.st));
+    RR_CUDA(cudaStreamSynchronize(S.st));
+    for (int32_t c : count) most += c;
+    const size_t off = ru((size_t)most * 8);
+    if ((s = grow(ix->outgrown, off + (size_t)most * 4, 0, S.st)) != RR_OK) return s;
+    uint64_t *key = (uint64_t *)ix->outgrown.p;
+    int32_t *slot = (int32_t *)((uint8_t *)ix->outgrown.p + off);
+    RR_CUDA(cudaMemcpyAsync(key, ho.key, (size_t)ho.count * 8, cudaMemcpyDeviceToDevice, S.st));
+    RR_CUDA(cudaMemcpyAsync(slot, ho.slot, (size_t)ho.count * 4, cudaMemcpyDeviceToDevice, S.st));
+    // the number of pending items, without the count of handed-over queries beside it, is the cursor
+    RR_CUDA(cudaMemsetAsync(S.counters + kCtrPend + 1, 0, 4, S.st));
+    if ((s = launch_gather_slots(g.item_key, g.item_slot, ho.tail, out, key, slot, most, g.hand_pend, S.st)) != RR_OK) return s;
+    ho.key = key;
+    ho.slot = slot;
+    ho.count = most;
+    return RR_OK;
+}
 
 // Alg. 2 for the queued queries, a cluster of CTAs each (k_bfs.cuh), and the scan of the final counts; their number
 // is read back only after both.  Queries handed over by the kernel are finished by the two-pass levels.  An item list
 // that was too short is grown to what the run has counted, and the kernel runs again (2,048 queries with 36 M results:
 // 9.2 ms a run, the level kernels, which grow the list as they go, 18.3).  If the results exceed max_results_total, or
-// a frontier or a handed-over query found no room, all queries are redone by the level kernels, which cut the results
-// at the cap.
+// more frontiers outgrew their lists than can be handed over, all queries are redone by the level kernels, which cut
+// the results at the cap.
 rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go) {
     rr_index *ix = S.ix;
     const SearchArgs &a = S.a;
@@ -428,10 +456,10 @@ rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go)
     g.np2 = S.counters + kCtrP2;
     g.next = S.counters + kCtrBfsNext;
     g.done = S.counters + kCtrBfsDone;
-    g.handed = S.counters + kCtrHand;
     g.overflow = S.counters + kCtrOverflow;
     g.levels = S.counters + kCtrLevels;
-    g.pend_count = (uint32_t *)(S.counters + kCtrPend);
+    g.hand_pend = (unsigned long long *)(S.counters + kCtrPend);
+    g.outgrown = S.counters + kCtrOutgrown;
     g.tail = S.tail;
     g.results = (unsigned long long *)(S.counters + kCtrResults);
     g.max_results = S.P.max_results_total;
@@ -471,9 +499,14 @@ rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go)
     }
     S.phase2_steps = S.hc[kCtrLevels];
     go.nitems = tail;
-    if (!capped && S.hc[kCtrHand] > 0) {
-        const HandOver ho{g.pend_key, g.pend_slot, (int64_t)(uint32_t)S.hc[kCtrPend], g.hand_bits, tail, results};
-        note_form(kFormHanded, S.hc[kCtrHand]);
+    const int32_t handed = S.hc[kCtrPend + 1];
+    if (!capped && handed > 0) {
+        HandOver ho{g.pend_key, g.pend_slot, (int64_t)(uint32_t)S.hc[kCtrPend], g.hand_bits, tail, results};
+        SlotList out{};
+        for (int h = 0; h < kHandCap; h++)
+            if (S.hc[kCtrOutgrown + h]) out.slot1[out.n++] = S.hc[kCtrOutgrown + h];
+        if (out.n > 0 && (s = take_outgrown(S, g, out, ho)) != RR_OK) return s;
+        note_form(kFormHanded, handed);
         if ((s = run_greedy(S, *np2, &ho, go, &capped)) != RR_OK) return s;
     }
     if (capped && (s = run_greedy(S, *np2, nullptr, go, &capped)) != RR_OK) return s;

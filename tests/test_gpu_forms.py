@@ -1,5 +1,6 @@
 """Which form of a phase a call takes (rr_debug_count), and each form against the CPU oracle, bit for bit, at the sizes
 where the other one is the library's choice next door."""
+import functools
 import os
 
 import numpy as np
@@ -89,6 +90,7 @@ def test_cap_counts_results_not_list_entries(rr):
     gi.close()
 
 
+@functools.lru_cache(maxsize=1)
 def _all_in_range(n, m, R, nq, seed):
     """m of n points joined by a random graph, a radius that holds all of them: every query's results are all m."""
     rng = np.random.default_rng(seed)
@@ -146,4 +148,22 @@ def test_a_capped_call_does_not_expand_everything_first(rr):
     assert np.all((res.flags & rr.RR_FLAG_TRUNCATED) != 0)
     assert capped < full, (capped, full)  # both forms one after the other took longer than the full expansion
     _check_all(gi.range_search(Q, 1e9, "greedy", beam=16), X, live, Q)
+    gi.close()
+
+
+@pytest.mark.parametrize("dtype", ["u8", "f32"])
+@pytest.mark.parametrize("nq", [1, 40])
+def test_frontier_that_outgrows_its_list_is_handed_over(rr, dtype, nq):
+    """From 16 points by rows of 128 the second level holds most of 400,000 points, above the list's 131,072 entries.
+    One such query is finished by the level kernels and nothing is done twice; 40 find no room there and are redone."""
+    X, adj, live, Q = _all_in_range(420_000, 400_000, 128, 40, 5)
+    Q = Q[:nq]
+    if dtype == "f32":
+        X, Q = X.astype(np.float32), Q.astype(np.float32)
+    gi = rr.Index.from_arrays(X, adj, 0)
+    handed, levels = rr.rr_debug_count("greedy_handed"), rr.rr_debug_count("greedy_levels")
+    res = gi.range_search(Q, 1e9, "greedy", beam=16)
+    assert rr.rr_debug_count("greedy_handed") == handed + (1 if nq == 1 else 0)
+    assert rr.rr_debug_count("greedy_levels") == levels + (0 if nq == 1 else 1)
+    _check_all(res, X, live, Q)
     gi.close()
