@@ -29,7 +29,7 @@ bool bfs_shape(int64_t n, int64_t nq, BfsShape *s) {
     return true;
 }
 
-size_t bfs_front_bytes(const BfsShape &s) { return (size_t)s.clusters * 2 * s.fcap * 4; }
+size_t bfs_front_bytes(const BfsShape &s) { return (size_t)2 * s.fcap * 4; }
 
 int64_t bfs_list_slack(const BfsShape &s) {
     return ((int64_t)s.clusters << s.cl_log2) * (s.threads / 32) * kBfsChunk;

@@ -253,7 +253,7 @@ struct BfsArgs {
 };
 // false: the index is too large for the bitmaps, the two-pass levels are the faster ones
 bool bfs_shape(int64_t n, int64_t nq, BfsShape *s);
-size_t bfs_front_bytes(const BfsShape &s);
+size_t bfs_front_bytes(const BfsShape &s);  // of one cluster
 // entries of the item list without an item, at most (a warp reserves whole chunks)
 int64_t bfs_list_slack(const BfsShape &s);
 rr_status launch_bfs(BfsArgs g, const BfsShape &s, cudaStream_t st, int dtype_code);

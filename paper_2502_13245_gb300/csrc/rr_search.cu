@@ -430,25 +430,63 @@ rr_status take_outgrown(Search &S, const BfsArgs &g, const SlotList &out, HandOv
     return RR_OK;
 }
 
+// Scratch that a batch takes before it knows of a queued query: reading their number first costs a host round trip
+// (about 10 us), which only batches that would take more than this pay, and these once they hold what they need no more.
+constexpr size_t kBfsOutright = (size_t)96 << 20;
+
+rr_status read_queued(Search &S, int32_t *np2) {
+    RR_CUDA(cudaMemcpyAsync(S.hc, S.a.p2_count, 4, cudaMemcpyDeviceToHost, S.st));
+    RR_CUDA(cudaStreamSynchronize(S.st));
+    *np2 = S.hc[0];
+    return RR_OK;
+}
+
 // Alg. 2 for the queued queries, a cluster of CTAs each (k_bfs.cuh), and the scan of the final counts; their number
 // is read back only after both.  Queries handed over by the kernel are finished by the two-pass levels.  An item list
 // that was too short is grown to what the run has counted, and the kernel runs again (2,048 queries with 36 M results:
 // 9.2 ms a run, the level kernels, which grow the list as they go, 18.3).  If the results exceed max_results_total, or
 // more frontiers outgrew their lists than can be handed over, all queries are redone by the level kernels, which cut
 // the results at the cap.
-rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go) {
+rr_status run_bfs(Search &S, BfsShape shape, int32_t *np2, GreedyOut &go) {
     rr_index *ix = S.ix;
     const SearchArgs &a = S.a;
     const int64_t words = (ix->n + 31) / 32;
     rr_status s;
-    const int64_t slack = bfs_list_slack(shape);
-    int64_t want = std::min<int64_t>(result_cap(S, S.nq), (int64_t)1 << 22) + slack;
+    // Scratch.  A batch that the lists held, or kBfsOutright, give half of the clusters that it could use goes without
+    // the number of queued queries; any other reads it first, takes nothing when it is 0 and lists for as many queries.
+    const size_t front1 = bfs_front_bytes(shape);
+    const int full = shape.clusters, have = (int)std::min<size_t>(full, ix->front.bytes / front1);
+    auto hand_bytes = [&](int64_t nq, int64_t *cap, size_t *off_pk, size_t *off_ps) {
+        const int64_t h = std::min<int64_t>(kHandCap, nq);
+        *cap = std::min<int64_t>(kPendCap, h * ix->n);
+        *off_pk = ru((size_t)h * words * 4);
+        *off_ps = *off_pk + ru((size_t)*cap * 8);
+        return *off_ps + (size_t)*cap * 4;
+    };
+    const int64_t slack = bfs_list_slack(shape);  // with all the clusters, which a later call may have
+    int64_t queued = S.nq, pend_cap;  // at most
+    size_t off_pk, off_ps, hand = hand_bytes(queued, &pend_cap, &off_pk, &off_ps);
+    shape.clusters = std::max(have, (full + 1) / 2);
+    const size_t more = (ix->front.bytes >= shape.clusters * front1 ? 0 : shape.clusters * front1) +
+                        (ix->hand.bytes >= hand ? 0 : hand);
+    const bool known = more > kBfsOutright;
+    if (known) {
+        if ((s = read_queued(S, np2)) != RR_OK) return s;
+        if (*np2 == 0) return RR_OK;
+        queued = *np2;
+        shape.clusters = (int)std::min<int64_t>(full, queued);
+        hand = hand_bytes(queued, &pend_cap, &off_pk, &off_ps);
+    }
+    int64_t want = std::min<int64_t>(result_cap(S, queued), known ? (int64_t)1 << 22 : (int64_t)1 << 20) + slack;
     if ((s = grow(ix->item_key, (size_t)want * 8, 0, S.st)) != RR_OK) return s;
     if ((s = grow(ix->item_slot, (size_t)want * 4, 0, S.st)) != RR_OK) return s;
-    if ((s = grow(ix->front, bfs_front_bytes(shape), 0, S.st)) != RR_OK) return s;
-    const uint32_t pend_cap = (uint32_t)std::min<int64_t>(kPendCap, kHandCap * ix->n);
-    const size_t off_pk = ru((size_t)kHandCap * words * 4), off_ps = off_pk + ru((size_t)pend_cap * 8);
-    if ((s = grow(ix->hand, off_ps + (size_t)pend_cap * 4, 0, S.st)) != RR_OK) return s;
+    if ((s = grow(ix->front, shape.clusters * front1, 0, S.st)) == RR_OK) s = grow(ix->hand, hand, 0, S.st);
+    if (s == RR_ENOMEM) {  // the level kernels need a bitmap a query, no more
+        if (!known && (s = read_queued(S, np2)) != RR_OK) return s;
+        bool capped;
+        return *np2 > 0 ? run_greedy(S, *np2, nullptr, go, &capped) : RR_OK;
+    }
+    if (s != RR_OK) return s;
     BfsArgs g;
     memset(&g, 0, sizeof g);
     g.s = a;
@@ -469,8 +507,8 @@ rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go)
     g.bail_total = kHandTotal;
     g.bail_front = kHandFront;
     g.bail_slots = kHandSlots >> shape.cl_log2;
-    g.hand_cap = kHandCap;
-    g.pend_cap = pend_cap;
+    g.hand_cap = (int32_t)std::min<int64_t>(kHandCap, queued);
+    g.pend_cap = (uint32_t)pend_cap;
     g.hand_of = S.hand_of;
     g.hand_bits = (uint32_t *)ix->hand.p;
     g.hand_words = words;
@@ -491,7 +529,8 @@ rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go)
         *np2 = S.hc[kCtrP2];
         capped = S.hc[kCtrOverflow] != 0 || results > result_cap(S, *np2);  // a run that stopped: overflow
         if (capped || tail <= g.cap) break;
-        want = results + slack;
+        // queries that this run handed over may be expanded further by the next
+        want = std::min<int64_t>(S.hc[kCtrPend + 1] > 0 ? 2 * results : results, result_cap(S, *np2)) + slack;
         if ((s = grow(ix->item_key, (size_t)want * 8, 0, S.st)) != RR_OK) return s;
         if ((s = grow(ix->item_slot, (size_t)want * 4, 0, S.st)) != RR_OK) return s;
         RR_CUDA(cudaMemsetAsync(S.counters + kCtrBfsNext, 0, (kCtrWords - kCtrBfsNext) * 4, S.st));
@@ -499,6 +538,8 @@ rr_status run_bfs(Search &S, const BfsShape &shape, int32_t *np2, GreedyOut &go)
     }
     S.phase2_steps = S.hc[kCtrLevels];
     go.nitems = tail;
+    // more queries than clusters: the next such batch has them (a failure leaves the lists as they are)
+    if (*np2 > shape.clusters && shape.clusters < full) grow(ix->front, std::min(full, *np2) * front1, 0, S.st);
     const int32_t handed = S.hc[kCtrPend + 1];
     if (!capped && handed > 0) {
         HandOver ho{g.pend_key, g.pend_slot, (int64_t)(uint32_t)S.hc[kCtrPend], g.hand_bits, tail, results};
@@ -759,9 +800,7 @@ extern "C" rr_status rr_range_search(rr_index *ix, const void *queries, int64_t 
     if (bfs) {
         if ((s = run_bfs(S, shape, &np2, go)) != RR_OK) return S.fail(s);
     } else if (a.phase2 && nq > 0) {
-        RR_CUDA(cudaMemcpyAsync(S.hc, a.p2_count, 4, cudaMemcpyDeviceToHost, S.st));
-        RR_CUDA(cudaStreamSynchronize(S.st));
-        np2 = S.hc[0];
+        if ((s = read_queued(S, &np2)) != RR_OK) return S.fail(s);
     }
     if (greedy && !bfs && np2 > 0) {
         bool capped;

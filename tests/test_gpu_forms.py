@@ -167,3 +167,47 @@ def test_frontier_that_outgrows_its_list_is_handed_over(rr, dtype, nq):
     assert rr.rr_debug_count("greedy_levels") == levels + (0 if nq == 1 else 1)
     _check_all(res, X, live, Q)
     gi.close()
+
+
+def test_scratch_of_the_expansion_is_not_taken_before_a_query_needs_it(rr):
+    """400 queries of a 3-megabyte index without a result: the search holds its arena and staging, no more."""
+    rng = np.random.default_rng(6)
+    n, R = 200_000, 4
+    X = rng.integers(0, 200, size=(n, 8), dtype=np.uint8)
+    gi = rr.Index.from_arrays(X, _graph(rng, n, R), 0)
+    Q = rng.integers(0, 200, size=(400, 8), dtype=np.uint8)
+    res = gi.range_search(Q, -1.0, "greedy", beam=16)
+    assert len(res.ids) == 0
+    assert rr.rr_index_info_get(gi.h).scratch_bytes < 32 << 20
+    gi.close()
+
+
+@pytest.mark.parametrize("dtype,d", [("u8", 16), ("u8", 32), ("i8", 48), ("u8", 64), ("i8", 200), ("u8", 512), ("f32", 24)])
+@pytest.mark.parametrize("R", [24, 32, 64, 97, 128])
+def test_level_kernels_where_the_clusters_find_no_scratch(rr, dtype, d, R):
+    """The expansion's own scratch (frontier lists, hand-over) does not fit: the level kernels take the batch, at every
+    split of a vector over lanes, by rows (degrees that are multiples of 32) and by pairs."""
+    rng = np.random.default_rng(d + R)
+    n, nq = 1500, 40
+    X = rng.integers(0, 30, size=(n, d)).astype({"u8": np.uint8, "i8": np.int8, "f32": np.float32}[dtype])
+    Q = rng.integers(0, 30, size=(nq, d)).astype(X.dtype)
+    d2 = ((X[None].astype(np.int64) - Q[:, None].astype(np.int64)) ** 2).sum(-1)
+    r = float(np.percentile(d2, 10))
+    adj = _graph(rng, n, R)
+    oi = oracle.Index(X, adj, 0)
+    o_ids, o_d, _ = oracle.range_search(oi, Q, r, "greedy", beam=8, threads=os.cpu_count() or 4)
+    assert sum(len(x) for x in o_ids) > nq * 8
+    for nth in (3, 4):  # after the arena and the item list: the frontier lists, then the hand-over buffer
+        gi = rr.Index.from_arrays(X, adj, 0)
+        levels = rr.rr_debug_count("greedy_levels")
+        try:
+            rr.rr_debug_set("fail_alloc_after", nth)
+            res = gi.range_search(Q, r, "greedy", beam=8)
+        finally:
+            rr.rr_debug_set("fail_alloc_after", -1)
+        assert rr.rr_debug_count("greedy_levels") == levels + 1
+        _same(res, o_ids, o_d)
+        cluster = rr.rr_debug_count("greedy_cluster")
+        _same(gi.range_search(Q, r, "greedy", beam=8), o_ids, o_d)
+        assert rr.rr_debug_count("greedy_cluster") == cluster + 1
+        gi.close()
