@@ -459,7 +459,8 @@ rr_status rr_debug_set(const char *key, int64_t value);
  *   "greedy_cluster"           greedy phases by a cluster of CTAs per query
  *   "greedy_again"             of these, run a second time with a longer list
  *   "greedy_handed"            queries these handed to the level kernels
- *   "greedy_levels"            greedy phases by the level kernels from the start */
+ *   "greedy_levels"            greedy phases by the level kernels from the start
+ *   "bin_sort", "segment_sort" sorts of greedy, doubling or 8-bit exhaustive results */
 int64_t rr_debug_count(const char *key);
 
 #ifdef __cplusplus

@@ -286,7 +286,8 @@ rr_status deliver(Search &S, int64_t total, uint32_t *ids, void *dists, rr_resul
 constexpr int64_t kBinSortItems = 8192;
 
 struct GreedyOut {
-    int64_t nitems = 0;
+    int64_t nitems = 0;    // entries of the item list, empty ones among them
+    int64_t nresults = 0;
 };
 
 // Queries that the cluster kernel handed to the two-pass levels: their pending items, bitmaps, the item list's end and
@@ -392,6 +393,7 @@ rr_status run_greedy(Search &S, int32_t np2, const HandOver *ho, GreedyOut &go, 
     }
     if (ho && *capped) return RR_OK;  // the caller starts over with every query
     go.nitems = tail;
+    go.nresults = tail - (ho ? ho->tail - ho->results : 0);
     S.total = -1;
     const int64_t from = ho ? init : 0;
     if (!ho) RR_CUDA(cudaMemsetAsync(g.slot_count, 0, (size_t)np2 * 4, S.st));
@@ -538,6 +540,7 @@ rr_status run_bfs(Search &S, BfsShape shape, int32_t *np2, GreedyOut &go) {
     }
     S.phase2_steps = S.hc[kCtrLevels];
     go.nitems = tail;
+    go.nresults = results;
     // more queries than clusters: the next such batch has them (a failure leaves the lists as they are)
     if (*np2 > shape.clusters && shape.clusters < full) grow(ix->front, std::min(full, *np2) * front1, 0, S.st);
     const int32_t handed = S.hc[kCtrPend + 1];
@@ -694,7 +697,7 @@ rr_status run_doubling(Search &S, int32_t np2, GreedyOut &go, bool warm) {
         b *= 2;
         first = false;
     }
-    go.nitems = (int64_t)tail_h;
+    go.nitems = go.nresults = (int64_t)tail_h;
     return launch_set_counts(S.a.res_count, S.flags, a.p2_list, S.slot_count, S.slot_trunc, np2, S.st);
 }
 
@@ -814,7 +817,8 @@ extern "C" rr_status rr_range_search(rr_index *ix, const void *queries, int64_t 
     uint32_t *ids = nullptr;
     void *dists = nullptr;
     const bool items = np2 > 0 && (greedy || doubling);
-    const bool bins = items && go.nitems >= kBinSortItems;
+    const bool bins = items && go.nresults >= kBinSortItems;
+    if (items) note_form(bins ? kFormBinSort : kFormSegmentSort);
     size_t bin_at = 0;
     if ((s = scan_and_alloc(S, &total, &ids, &dists, items ? 1 : 0, bins ? go.nitems : 0, np2, &bin_at)) != RR_OK)
         return S.fail(s);
@@ -886,6 +890,7 @@ static rr_status brute_8bit(Search &S, rr_result *out) {
     void *dists = nullptr;
     size_t bin_at = 0;
     const bool bins = S.total >= kBinSortItems;
+    note_form(bins ? kFormBinSort : kFormSegmentSort);
     if ((s = scan_and_alloc(S, &total, &ids, &dists, 1, bins ? S.total : 0, nq, &bin_at)) != RR_OK) return s;
     const OutArgs o{nq, S.offsets, 0, ids, dists, S.flags, total, a.error, nullptr};
     if (!bins) {

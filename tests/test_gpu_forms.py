@@ -211,3 +211,17 @@ def test_level_kernels_where_the_clusters_find_no_scratch(rr, dtype, d, R):
         _same(gi.range_search(Q, r, "greedy", beam=8), o_ids, o_d)
         assert rr.rr_debug_count("greedy_cluster") == cluster + 1
         gi.close()
+
+
+@pytest.mark.parametrize("n,form", [(1023, "segment_sort"), (1024, "bin_sort")])
+@pytest.mark.parametrize("call", ["greedy", "doubling", "brute"])
+def test_the_sort_is_chosen_by_results(rr, n, form, call):
+    """8 queries that hold every point: 8,184 and 8,192 results.  Empty entries of the cluster expansion's item list do
+    not count."""
+    X, adj, Q = _data(n, 8, 16, 8, n)
+    gi = rr.Index.from_arrays(X, adj, 0)
+    before = rr.rr_debug_count(form)
+    res = gi.brute_force(Q, 1e9) if call == "brute" else gi.range_search(Q, 1e9, call, beam=16)
+    assert rr.rr_debug_count(form) == before + 1
+    _check_all(res, X, np.arange(n), Q)
+    gi.close()
