@@ -351,7 +351,10 @@ rr_status run_greedy(Search &S, int32_t np2, const HandOver *ho, GreedyOut &go, 
     int64_t begin = 0, end = ho ? ho->count : init, tail = init, levels = 0;
     bool pending = ho != nullptr;
     *capped = false;
-    if (!ho) note_form(kFormLevels);
+    if (!ho) {
+        note_form(kFormLevels);
+        S.phase2_steps = 0;  // all that counts is done here
+    }
     while (begin < end) {
         const int64_t need = tail + (end - begin) * (int64_t)ix->R;
         if (need > g.cap && g.cap < cap_limit) {

@@ -225,3 +225,21 @@ def test_the_sort_is_chosen_by_results(rr, n, form, call):
     assert rr.rr_debug_count(form) == before + 1
     _check_all(res, X, np.arange(n), Q)
     gi.close()
+
+
+def test_steps_of_a_redone_phase(rr):
+    """rr_profile.phase2_steps of a capped call counts the levels that made the result, not those before it."""
+    X, adj, Q = _data(3000, 16, 20, 60, 8)
+    r = _radius(X, Q, 10)
+    steps = []
+    for nth in (-1, 3):  # the clusters first, then the level kernels; the level kernels only
+        gi = rr.Index.from_arrays(X, adj, 0)
+        try:
+            rr.rr_debug_set("fail_alloc_after", nth)
+            res = gi.range_search(Q, r, "greedy", beam=8, max_results_total=1000, profile=1)
+        finally:
+            rr.rr_debug_set("fail_alloc_after", -1)
+        assert res.status == rr.RR_EOVERFLOW
+        steps.append(rr.rr_last_profile(gi.h).phase2_steps)
+        gi.close()
+    assert steps[0] == steps[1] > 0
