@@ -460,7 +460,10 @@ rr_status rr_debug_set(const char *key, int64_t value);
  *   "greedy_again"             of these, run a second time with a longer list
  *   "greedy_handed"            queries these handed to the level kernels
  *   "greedy_levels"            greedy phases by the level kernels from the start
- *   "bin_sort", "segment_sort" sorts of greedy, doubling or 8-bit exhaustive results */
+ *   "bin_sort", "segment_sort" sorts of greedy, doubling or 8-bit exhaustive results
+ *   "brute_tensor"             exhaustive scans on the tensor cores (8-bit)
+ *   "brute_two_pass"           by a count and a fill pass (fp32; 8-bit where the
+ *                              tensor-core form's item list does not fit) */
 int64_t rr_debug_count(const char *key);
 
 #ifdef __cplusplus

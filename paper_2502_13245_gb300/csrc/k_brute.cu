@@ -1,5 +1,7 @@
 // k_brute.cu -- exact range search by exhaustive scan (Def. 2.1), the ground
-// truth against which average precision (Def. 2.2) is measured.
+// truth against which average precision (Def. 2.2) is measured: fp32 indexes, and
+// 8-bit ones where the item list of the tensor-core form (k_brute_tc.cu) does not
+// fit the device -- these two passes need the sort keys alone (8 bytes a match).
 //
 // A CTA takes QT queries (kept in shared memory) and 256 points (one per
 // thread, streamed from HBM in 16-byte chunks); every thread accumulates QT

@@ -19,7 +19,7 @@ rr_status cuda_fail(cudaError_t e, const char *what);
 rr_status allow_smem(const void *kernel, size_t bytes);
 // forms of the phases, counted for rr_debug_count
 enum Form { kFormBeamWarp, kFormBeamCta, kFormRoundWarp, kFormRoundCta, kFormCluster, kFormClusterAgain, kFormHanded, kFormLevels,
-            kFormBinSort, kFormSegmentSort, kForms };
+            kFormBinSort, kFormSegmentSort, kFormBruteTensor, kFormBruteTwoPass, kForms };
 void note_form(Form f, int64_t k = 1);
 // failure-path hooks set by rr_debug_set: true if this device allocation is to fail;
 // the beam and doubling kernels' per-query iteration guard (default n + 1); the tries of a wait in the 8-bit

@@ -71,7 +71,7 @@ static std::atomic<int64_t> g_brute_wait_tries{-1};
 static std::atomic<int64_t> g_forms[kForms];
 static const char *const kFormKeys[kForms] = {"beam_warp", "beam_cta", "round_warp", "round_cta",
                                              "greedy_cluster", "greedy_again", "greedy_handed", "greedy_levels",
-                                             "bin_sort", "segment_sort"};
+                                             "bin_sort", "segment_sort", "brute_tensor", "brute_two_pass"};
 
 void note_form(Form f, int64_t k) { g_forms[f].fetch_add(k, std::memory_order_relaxed); }
 

@@ -204,9 +204,20 @@ rr_status scan_counts(Search &S) {
     return RR_OK;
 }
 
+// The staging buffer: `end` bytes and the bin sort's scratch behind them.
+rr_status grow_output(Search &S, size_t end, int64_t bin_items, int64_t bin_slots, size_t *bin_at) {
+    *bin_at = bin_items ? end : 0;
+    if (bin_items) {
+        const rr_status s = grow(S.ix->outbuf, bin_sort_end(bin_items, bin_slots, end), 0, S.st);
+        if (s != RR_ENOMEM) return s;
+        *bin_at = 0;
+    }
+    return grow(S.ix->outbuf, end, 0, S.st);
+}
+
 // Allocate the id/dist arrays for the final per-query counts.
 // extra_keys: also room for total sort keys at the start of the staging buffer; bin_items, bin_slots: and for the
-// bin sort's scratch, at *bin_at.
+// bin sort's scratch, at *bin_at (0: none asked for, or it does not fit, then the sort of segments needs none).
 rr_status scan_and_alloc(Search &S, int64_t *total, uint32_t **ids, void **dists, size_t extra_keys,
                          int64_t bin_items, int64_t bin_slots, size_t *bin_at) {
     rr_index *ix = S.ix;
@@ -218,17 +229,11 @@ rr_status scan_and_alloc(Search &S, int64_t *total, uint32_t **ids, void **dists
         *ids = (uint32_t *)S.res_alloc(t * 4);
         *dists = S.res_alloc(t * 4);
         if (!*ids || !*dists) { set_error("result allocation failed"); return RR_ENOMEM; }
-        size_t end = extra_keys ? ru(t * 8) : 256;
-        *bin_at = end;
-        if (bin_items) end = bin_sort_end(bin_items, bin_slots, end);
-        if ((s = grow(ix->outbuf, end, 0, S.st)) != RR_OK) return s;
+        if ((s = grow_output(S, extra_keys ? ru(t * 8) : 256, bin_items, bin_slots, bin_at)) != RR_OK) return s;
     } else {
         // staging: [sort keys: t x 8][ids: t x 4][dists: t x 4], each region 256-byte aligned
         const size_t off_ids = ru(t * 8), off_d = off_ids + ru(t * 4);
-        size_t end = off_d + ru(t * 4);
-        *bin_at = end;
-        if (bin_items) end = bin_sort_end(bin_items, bin_slots, end);
-        if ((s = grow(ix->outbuf, end, 0, S.st)) != RR_OK) return s;
+        if ((s = grow_output(S, off_d + ru(t * 4), bin_items, bin_slots, bin_at)) != RR_OK) return s;
         *ids = (uint32_t *)((uint8_t *)ix->outbuf.p + off_ids);
         *dists = (uint8_t *)ix->outbuf.p + off_d;
     }
@@ -820,11 +825,12 @@ extern "C" rr_status rr_range_search(rr_index *ix, const void *queries, int64_t 
     uint32_t *ids = nullptr;
     void *dists = nullptr;
     const bool items = np2 > 0 && (greedy || doubling);
-    const bool bins = items && go.nresults >= kBinSortItems;
-    if (items) note_form(bins ? kFormBinSort : kFormSegmentSort);
     size_t bin_at = 0;
-    if ((s = scan_and_alloc(S, &total, &ids, &dists, items ? 1 : 0, bins ? go.nitems : 0, np2, &bin_at)) != RR_OK)
+    if ((s = scan_and_alloc(S, &total, &ids, &dists, items ? 1 : 0,
+                            items && go.nresults >= kBinSortItems ? go.nitems : 0, np2, &bin_at)) != RR_OK)
         return S.fail(s);
+    const bool bins = bin_at > 0;
+    if (items) note_form(bins ? kFormBinSort : kFormSegmentSort);
     OutArgs o{nq, S.offsets, ix->dtype == RR_F32 ? 1 : 0, ids, dists, S.flags, total, S.a.error, ix->ext};
     if ((s = launch_copy_slots(o, a.res_keys, a.beam, a.res_count, nullptr, (int32_t)nq, S.st)) != RR_OK) return S.fail(s);
     if (bins) {
@@ -868,6 +874,7 @@ extern "C" rr_status rr_range_search(rr_index *ix, const void *queries, int64_t 
 // Def. 2.1 for an 8-bit index (k_brute_tc.cu): one pass over all pairs into the item list, then the bin sort.  A list
 // that was too small is grown to the counted total and the pass repeated.
 static rr_status brute_8bit(Search &S, rr_result *out) {
+    note_form(kFormBruteTensor);
     rr_index *ix = S.ix;
     SearchArgs &a = S.a;
     const int64_t nq = S.nq;
@@ -892,9 +899,10 @@ static rr_status brute_8bit(Search &S, rr_result *out) {
     uint32_t *ids = nullptr;
     void *dists = nullptr;
     size_t bin_at = 0;
-    const bool bins = S.total >= kBinSortItems;
+    if ((s = scan_and_alloc(S, &total, &ids, &dists, 1, S.total >= kBinSortItems ? S.total : 0, nq, &bin_at)) != RR_OK)
+        return s;
+    const bool bins = bin_at > 0;
     note_form(bins ? kFormBinSort : kFormSegmentSort);
-    if ((s = scan_and_alloc(S, &total, &ids, &dists, 1, bins ? S.total : 0, nq, &bin_at)) != RR_OK) return s;
     const OutArgs o{nq, S.offsets, 0, ids, dists, S.flags, total, a.error, nullptr};
     if (!bins) {
         uint64_t *tmp = (uint64_t *)ix->outbuf.p;  // a.p2_list (zeroed) is the cursor of each segment
@@ -938,9 +946,23 @@ extern "C" rr_status rr_brute_force(rr_index *ix, const void *queries, int64_t n
     SearchArgs &a = S.a;
     a.ext = ix->ext;  // keys carry the caller's ids, so the sort below is by (distance, id)
     if (nq > 0 && brute_tc(ix->dtype)) {
+        const size_t held = S.owned.size();
         s = brute_8bit(S, out);
-        return s == RR_OK ? RR_OK : S.fail(s);
+        if (s == RR_OK) return RR_OK;
+        if (s != RR_ENOMEM) return S.fail(s);
+        // the item list (12 bytes a match beside the keys) does not fit: two passes without one
+        while (S.owned.size() > held) {
+            cudaFreeAsync(S.owned.back(), S.st);
+            S.owned.pop_back();
+        }
+        RR_CUDA(cudaStreamSynchronize(S.st));
+        grow_free(ix->item_key);
+        grow_free(ix->item_slot);
+        S.total = -1;
+        RR_CUDA(cudaMemsetAsync(a.res_count, 0, (size_t)nq * 4, S.st));
+        RR_CUDA(cudaMemsetAsync(a.p2_list, 0, (size_t)nq * 4, S.st));
     }
+    if (nq > 0) note_form(kFormBruteTwoPass);
     int32_t *counts = a.res_count, *cursor = a.p2_list;
     if ((s = launch_brute(a, counts, nullptr, nullptr, nullptr, 0, S.st, ix->dtype)) != RR_OK) return S.fail(s);
     int64_t total = 0;

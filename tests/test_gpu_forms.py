@@ -243,3 +243,42 @@ def test_steps_of_a_redone_phase(rr):
         steps.append(rr.rr_last_profile(gi.h).phase2_steps)
         gi.close()
     assert steps[0] == steps[1] > 0
+
+
+@pytest.mark.parametrize("dtype", ["u8", "i8"])
+@pytest.mark.parametrize("metric", ["l2", "ip"])
+@pytest.mark.parametrize("on_device", [False, True])
+def test_exhaustive_scan_whose_scratch_does_not_fit(rr, dtype, metric, on_device):
+    """Without room for the item list the two passes run, without room for the bins the sort of segments; what fits
+    the results and their keys still runs."""
+    rng = np.random.default_rng(9)
+    n, nq, d = 3000, 40, 100
+    X = rng.integers(0, 100, size=(n, d)).astype(np.uint8 if dtype == "u8" else np.int8)
+    Q = rng.integers(0, 100, size=(nq, d)).astype(X.dtype)
+    x, q = X.astype(np.int64), Q.astype(np.int64)
+    D = -(q @ x.T) if metric == "ip" else (q * q).sum(1)[:, None] + (x * x).sum(1)[None] - 2 * (q @ x.T)
+    r = float(np.percentile(D, 30))
+    assert (D <= r).sum() >= 8192
+    adj = np.full((n, 2), 0xFFFFFFFF, np.uint32)
+    first = 3 if on_device else 1  # after the arena (and the device result's offsets and flags)
+    bins = first + (4 if on_device else 2)  # after the item list (and the ids and distances)
+    for nth, form in ((first, "brute_two_pass"), (first + 1, "brute_two_pass"), (bins, "segment_sort"), (-1, "bin_sort")):
+        gi = rr.Index.from_arrays(X, adj, 0, metric=rr.RR_IP if metric == "ip" else rr.RR_L2)
+        before = rr.rr_debug_count(form)
+        try:
+            rr.rr_debug_set("fail_alloc_after", nth)
+            res = rr.rr_brute_force(gi.h, Q, r, result_on_device=on_device)
+        finally:
+            rr.rr_debug_set("fail_alloc_after", -1)
+        assert rr.rr_debug_count(form) == before + 1, (nth, form)
+        if on_device:
+            host = rr.rr_result_to_host(res)
+            rr.rr_result_free(res)
+            res = host
+        res = rr.RangeResult(res)
+        for i in range(nq):
+            ids = np.nonzero(D[i] <= r)[0]
+            o = np.lexsort((ids, D[i][ids]))
+            g_ids, g_d = res.query(i)
+            assert np.array_equal(g_ids, ids[o]) and np.array_equal(g_d, D[i][ids[o]]), (nth, i)
+        gi.close()
