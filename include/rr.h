@@ -96,11 +96,14 @@ typedef struct {
     double es_radius;          /* Alg. 5 esr when es_radius_mode = 1 */
     int32_t precision;         /* rr_precision (fp32 indexes only) */
     float recheck_eps;         /* low-precision slack: recheck when approx <= r + eps*|r| (0 = derive) */
-    int32_t persistent;        /* 1: one persistent launch with a device work queue */
+    int32_t persistent;        /* 1: one persistent launch with a device work queue (see tile_hint) */
     int32_t collect_stats;     /* 1: fill rr_result.stats (exact visit / distinct-id counts) */
     int64_t max_results_total; /* cap on the summed results of the greedy / doubling phase (0 = default
                                   1<<28); each query's first beam (at most b results) is always kept */
-    int32_t tile_hint;         /* warps per CTA for the beam kernel (0 = library choice) */
+    int32_t tile_hint;         /* warps per CTA for the beam kernel (0 = library choice).  tile_hint and persistent
+                                  shape the launch with a warp per query.  Batches of at most 1,216 queries with
+                                  beam >= 32 go by a CTA per query, of a size that the library chooses, and take
+                                  neither: exact precision, expand <= 1, no stats, es_metric d_visited or d_top1 */
     int32_t profile;           /* 1: record per-phase device times, see rr_last_profile */
     int32_t seen_log2;         /* log2 slots of the beam kernel's seen table, 5..14 (0 = library choice) */
     int32_t es_metric;         /* the M of Alg. 4 (Sec. 3.2), see rr_es_metric; RR_ES_VISITED is Alg. 5 */
@@ -314,8 +317,8 @@ rr_status rr_last_profile(rr_index *index, rr_profile *out);
  *   radius      one radius for every query (metric units)
  *   variant     RR_BEAM or RR_BEAM_ES; params may be NULL (defaults; b <= 512).
  *               The beam, the early-stop settings (every rr_es_metric) and the
- *               launch shape (tile_hint, seen_log2, persistent) are honoured as
- *               in rr_range_search; precision must be RR_PREC_EXACT (the
+ *               launch shape (tile_hint, seen_log2, persistent) are taken as in
+ *               rr_range_search; precision must be RR_PREC_EXACT (the
  *               low-precision copies are allocated on first use): RR_EINVAL
  *               otherwise
  *   out_counts  nq int32 (device): |N| of each query

@@ -9,7 +9,8 @@ queries from a device counter, versus one warp per query in a full grid).  `tune
 on the caller's batch with CUDA events, re-times the three fastest and the library default in interleaved
 rounds, and keeps a non-default setting only if its median beats the default's by more than 2% (single
 timings of a few-millisecond batch differ by more than the settings do); results are cached per (index
-shape, beam, variant).
+shape, beam, variant).  Batches that go by a CTA per query (`shape_matters`) have no launch shape to tune: they get the
+library's choice, and nothing is cached for the larger batches of the same index.
 """
 from __future__ import annotations
 
@@ -20,6 +21,7 @@ import os
 TILES = (2, 4, 8)
 SEEN_LOG2 = (9, 10, 11)
 PERSISTENT = (0, 1)
+BEAM_CTA_QUERIES, BEAM_CTA_BEAM = 1216, 32  # csrc/rr_internal.h, csrc/k_beam_cta.cu
 
 
 def choose(runs, default, margin=0.98):
@@ -33,6 +35,15 @@ def choose(runs, default, margin=0.98):
     return best, med
 
 
+def shape_matters(nq, beam, variant, params=None):
+    """False for the batches that the library searches with a CTA per query, whatever the shape (include/rr.h,
+    rr_params.tile_hint)."""
+    p = dict(params or {})
+    small = nq <= BEAM_CTA_QUERIES and beam >= BEAM_CTA_BEAM
+    plain = not p.get("precision") and p.get("expand", 0) <= 1 and not p.get("collect_stats")
+    return not (small and plain and (not variant.endswith("_es") or p.get("es_metric", 0) in (0, 1)))
+
+
 def _key(info, variant, beam):
     return "n%d_d%d_R%d_dt%d_%s_b%d" % (info.n, info.d, info.R, info.dtype, variant, beam)
 
@@ -42,6 +53,8 @@ def tune(index, queries, radius, variant, beam, stream=None, reps=3, cache_path=
     import torch
 
     import paper_2502_13245_gb300 as rr
+    if not shape_matters(queries.shape[0], beam, variant, base_params):
+        return {"tile_hint": 0, "seen_log2": 0, "persistent": 0}, []
     key = _key(index.info, variant, beam)
     cache = {}
     if cache_path and os.path.exists(cache_path):

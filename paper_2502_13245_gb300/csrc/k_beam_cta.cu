@@ -27,7 +27,7 @@ namespace {
 
 constexpr int kMaxW = 8;  // warps of a CTA = parents of a step
 
-constexpr int kHashLg = 11;
+constexpr int kHashLg = 11;  // unless the caller sets seen_log2
 
 __host__ __device__ inline int even(int x) { return (x + 1) & ~1; }
 __host__ __device__ inline size_t cta_smem_bytes(int b, int R, int W, int hlg) {
@@ -263,9 +263,10 @@ template <int DT, int CPL>
 rr_status launch_t(const SearchArgs &a, cudaStream_t st) {
     auto k = beam_cta_kernel<DT, CPL>;
     const int W = a.nq <= kBeamCta8 ? 8 : (a.nq <= kBeamCta4 ? 4 : 2);
-    const size_t smem = cta_smem_bytes(a.beam, a.R, W, kHashLg);
+    const int hlg = a.hash_lg > 0 ? a.hash_lg : kHashLg;
+    const size_t smem = cta_smem_bytes(a.beam, a.R, W, hlg);
     if (rr_status e = allow_smem((const void *)k, smem)) return e;
-    k<<<(unsigned)a.nq, 32 * W, smem, st>>>(a, kHashLg);
+    k<<<(unsigned)a.nq, 32 * W, smem, st>>>(a, hlg);
     RR_CUDA(cudaGetLastError());
     note_launch();
     return RR_OK;
@@ -277,7 +278,7 @@ rr_status launch_t(const SearchArgs &a, cudaStream_t st) {
 // early stop that the lookahead can foresee, and beams long enough to have points in line (beam 16: 172 -> 186 us,
 // beam 64: 521 -> 400 us at 64 queries).
 bool beam_cta(const SearchArgs &a) {
-    return a.nq <= kBeamCta2 && a.beam >= 32 && a.expand <= 1 && !a.count_bits && !a.stats && a.prec == RR_PREC_EXACT &&
+    return a.nq <= kBeamCta2 && a.beam >= kBeamCtaBeam && a.expand <= 1 && !a.count_bits && !a.stats && a.prec == RR_PREC_EXACT &&
            (!a.use_es || a.es_metric == RR_ES_VISITED || a.es_metric == RR_ES_TOP1);
 }
 

@@ -26,7 +26,8 @@
 //
 // Parameters are those of rr_range_search for RR_BEAM / RR_BEAM_ES: the beam,
 // the Alg. 5 / Alg. 4 early-stop settings (every metric), the launch shape
-// (tile_hint, seen_log2, persistent); results are equal for equal settings.
+// (seen_log2; tile_hint and persistent where a warp takes a query); results are
+// equal for equal settings.
 // Low-precision traversal is refused (its traversal copies are allocated on
 // first use), as are per-query radii.
 #include <string.h>
