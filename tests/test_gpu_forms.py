@@ -282,3 +282,94 @@ def test_exhaustive_scan_whose_scratch_does_not_fit(rr, dtype, metric, on_device
             g_ids, g_d = res.query(i)
             assert np.array_equal(g_ids, ids[o]) and np.array_equal(g_d, D[i][ids[o]]), (nth, i)
         gi.close()
+
+
+def _tiled(res, nq, o_ids, o_d):
+    for i in range(nq):
+        ids, d = res.query(i)
+        assert np.array_equal(ids, o_ids[i % len(o_ids)]), i
+        assert np.array_equal(d.astype(np.int64), np.asarray(o_d[i % len(o_d)]).astype(np.int64)), i
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(persistent=1), dict(tile_hint=2, seen_log2=6), dict(tile_hint=8, seen_log2=12),
+                                dict(persistent=1, tile_hint=1, seen_log2=5), dict(expand=2), dict(persistent=1, expand=3)])
+@pytest.mark.parametrize("variant,beam", [("greedy_es", 32), ("beam", 64), ("beam_es", 129), ("greedy", 200), ("beam", 400)])
+def test_warp_form_in_every_launch_shape(rr, kw, variant, beam):
+    """More queries than the CTA form takes (1,216), with the padded arrays of long beams (129 and more) and without."""
+    X, adj, Q = _data(2000, 12, 40, 130, 10)
+    r = _radius(X, Q, 12)
+    gi, oi = rr.Index.from_arrays(X, adj, 0), oracle.Index(X, adj, 0)
+    o_ids, o_d, _ = oracle.range_search(oi, Q, r, variant, beam=beam, expand=kw.get("expand", 1),
+                                        threads=os.cpu_count() or 4)
+    before = rr.rr_debug_count("beam_warp")
+    res = gi.range_search(np.tile(Q, (10, 1)), r, variant, beam=beam, **kw)
+    assert rr.rr_debug_count("beam_warp") == before + 1
+    _tiled(res, 1300, o_ids, o_d)
+    gi.close()
+
+
+def _unit(rng, n, d):
+    X = rng.standard_normal((n, d)).astype(np.float32)
+    return X / np.linalg.norm(X, axis=1, keepdims=True)
+
+
+@pytest.mark.parametrize("d", [100, 200, 500])
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("beam", [100, 150, 500])
+def test_warp_form_fp32(rr, d, precision, beam):
+    """Float rows of one to four chunks a lane: the exact traversal against the CTA form, the low-precision ones against
+    the kernel that keeps exact counters."""
+    if precision == 1 and d > 256:
+        pytest.skip("BF16 traversal takes d <= 256")
+    rng = np.random.default_rng(d + beam)
+    X = _unit(rng, 2500, d)
+    Q = (X[rng.integers(0, len(X), 130)] + 0.02 * rng.standard_normal((130, d))).astype(np.float32)
+    gi = rr.Index.from_arrays(X, _graph(rng, len(X), 24), 0, metric=rr.RR_IP)
+    for variant in ("beam", "beam_es"):
+        kw = dict(beam=beam, precision=precision)
+        before = rr.rr_debug_count("beam_warp")
+        got = gi.range_search(np.tile(Q, (10, 1)), -0.1, variant, **kw)
+        assert rr.rr_debug_count("beam_warp") == before + 1
+        want = gi.range_search(Q, -0.1, variant, collect_stats=1 if precision else 0, **kw)
+        assert len(want.ids) > 0
+        for i in range(1300):
+            for g, w in zip(got.query(i), want.query(i % 130)):
+                assert np.array_equal(g, w), i
+    gi.close()
+
+
+@pytest.mark.parametrize("L", [129, 300])
+def test_construction_with_long_beams(rr, L):
+    import rrsynth
+    X = np.random.default_rng(L).integers(0, 100, size=(1200, 16), dtype=np.uint8)
+    want, start = rrsynth.build_graph(X, 12, L, 1.2, seed=3)
+    got, _ = rr.rr_build_graph(X, 12, L, 1.2, passes=2, seed=3, start=start, metric=rr.RR_L2)
+    assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("variant", ["doubling", "doubling_es", "doubling_warm", "doubling_warm_es"])
+@pytest.mark.parametrize("kind", ["u8", "u8_counters", "f32", "bf16", "fp8"])
+def test_doubling_rounds_by_a_warp_per_query(rr, variant, kind):
+    """More active queries than the CTA form takes (608); the same queries in small batches go by CTA."""
+    rng = np.random.default_rng(11)
+    n, d, nq = 900, 16, 650
+    if kind.startswith("u8"):
+        X = rng.integers(0, 30, size=(n, d), dtype=np.uint8)
+        Q = rng.integers(0, 30, size=(50, d), dtype=np.uint8)
+        r, metric = _radius(X, Q, 90), rr.RR_L2
+    else:
+        X = _unit(rng, n, d)
+        Q, r, metric = _unit(rng, 50, d), 0.3, rr.RR_IP
+    gi = rr.Index.from_arrays(X, _graph(rng, n, 12), 0, metric=metric)
+    kw = dict(beam=8, precision={"bf16": 1, "fp8": 2}.get(kind, 0), es_visit_limit=10**6)
+    cta = rr.rr_debug_count("round_cta")
+    want = gi.range_search(Q, r, variant, **kw)
+    assert rr.rr_debug_count("round_cta") > cta
+    warp = rr.rr_debug_count("round_warp")
+    got = gi.range_search(np.tile(Q, (13, 1)), r, variant, collect_stats=1 if kind == "u8_counters" else 0, **kw)
+    assert rr.rr_debug_count("round_warp") > warp
+    assert len(want.ids) > 50 * 8
+    for i in range(nq):
+        for g, w in zip(got.query(i), want.query(i % 50)):
+            assert np.array_equal(g, w), i
+    gi.close()
