@@ -101,9 +101,10 @@ typedef struct {
     int64_t max_results_total; /* cap on the summed results of the greedy / doubling phase (0 = default
                                   1<<28); each query's first beam (at most b results) is always kept */
     int32_t tile_hint;         /* warps per CTA for the beam kernel (0 = library choice).  tile_hint and persistent
-                                  shape the launch with a warp per query.  Batches of at most 1,216 queries with
-                                  beam >= 32 go by a CTA per query, of a size that the library chooses, and take
-                                  neither: exact precision, expand <= 1, no stats, es_metric d_visited or d_top1 */
+                                  shape the launch with a warp per query.  Small batches go by a CTA per query,
+                                  of a size that the library chooses, and take neither: beam >= 32 and at most 608
+                                  queries (1,216 up to beam 128, fp32 256), exact precision, expand <= 1, no stats,
+                                  es_metric d_visited or d_top1 */
     int32_t profile;           /* 1: record per-phase device times, see rr_last_profile */
     int32_t seen_log2;         /* log2 slots of the beam kernel's seen table, 5..14 (0 = library choice) */
     int32_t es_metric;         /* the M of Alg. 4 (Sec. 3.2), see rr_es_metric; RR_ES_VISITED is Alg. 5 */

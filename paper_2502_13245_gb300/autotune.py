@@ -21,7 +21,9 @@ import os
 TILES = (2, 4, 8)
 SEEN_LOG2 = (9, 10, 11)
 PERSISTENT = (0, 1)
-BEAM_CTA_QUERIES, BEAM_CTA_BEAM = 1216, 32  # csrc/rr_internal.h, csrc/k_beam_cta.cu
+# csrc/rr_internal.h, csrc/k_beam_cta.cu: most queries with long and with other beams, the shortest beam, and the
+# longest that are not long (8-bit, fp32)
+BEAM_CTA_QUERIES, BEAM_CTA_BEAM, BEAM_CTA_LONG = (608, 1216), 32, (128, 256)
 
 
 def choose(runs, default, margin=0.98):
@@ -35,11 +37,12 @@ def choose(runs, default, margin=0.98):
     return best, med
 
 
-def shape_matters(nq, beam, variant, params=None):
+def shape_matters(nq, beam, variant, params=None, fp32=False):
     """False for the batches that the library searches with a CTA per query, whatever the shape (include/rr.h,
     rr_params.tile_hint)."""
     p = dict(params or {})
-    small = nq <= BEAM_CTA_QUERIES and beam >= BEAM_CTA_BEAM
+    most = BEAM_CTA_QUERIES[1 if beam <= BEAM_CTA_LONG[1 if fp32 else 0] else 0]
+    small = nq <= most and beam >= BEAM_CTA_BEAM
     plain = not p.get("precision") and p.get("expand", 0) <= 1 and not p.get("collect_stats")
     return not (small and plain and (not variant.endswith("_es") or p.get("es_metric", 0) in (0, 1)))
 
@@ -53,7 +56,7 @@ def tune(index, queries, radius, variant, beam, stream=None, reps=3, cache_path=
     import torch
 
     import paper_2502_13245_gb300 as rr
-    if not shape_matters(queries.shape[0], beam, variant, base_params):
+    if not shape_matters(queries.shape[0], beam, variant, base_params, index.info.dtype == rr.RR_F32):
         return {"tile_hint": 0, "seen_log2": 0, "persistent": 0}, []
     key = _key(index.info, variant, beam)
     cache = {}

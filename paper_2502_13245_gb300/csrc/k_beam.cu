@@ -529,7 +529,7 @@ rr_status launch_beam(const SearchArgs &a, int wpc, cudaStream_t st, int dtype_c
         set_error("beam phase: seen-table size 2^%d out of [2^5, 2^14]", hlg);
         return RR_EINVAL;
     }
-    if (beam_cta(a)) {  // a small batch
+    if (beam_cta(a, dtype_code)) {  // a small batch
         note_form(kFormBeamCta);
         return launch_beam_cta(a, st, dtype_code);
     }

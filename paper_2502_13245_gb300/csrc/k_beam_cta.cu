@@ -14,9 +14,14 @@
 // written in another, and racing writers can only lose an id, which costs a repeated evaluation.
 //
 // Measured (GB300, beam phase, a warp per query -> this): 1 query, beam 192, 10^6 x 128 u8, R = 64: 175 -> 110 us.
-// 2*10^5 x 128 u8, R = 32, beam 64 / 192: 256 queries 523 / 1,150 -> 403 / 724 us (8 warps a query), 512 queries
-// 522 / 1,137 -> 420 / 821 us (4), 1,024 queries 528 / 1,299 -> 485 / 1,170 us (2).  At 2,048 queries a warp each
-// fills the chip: 651 / 1,317 us against 659 / 1,593.  Bound: the chain of steps (row, gather, six barriers).
+// By warps a query, on five indexes (u8 128 B, R = 64 and 128; i8 256 B, R = 24; fp32 800 B, R = 64, and 2 KB, R = 128),
+// beams 32 to 512, with and without early stop, the warp form's time over this one's:
+//   8 (up to 304 queries)    1.2 to 2.7 times up to beam 256, 1.0 to 2.1 beyond (1.0: 8-bit, one query)
+//   4 (305 to 608)           1.1 to 1.9; one of the cases loses: i8, early stop, beam 512, 0.94
+//   2 (609 to 1,216)         8-bit 1.02 to 1.21 up to beam 128, 0.92 to 1.04 at 160 to 256, 0.80 to 0.94 beyond;
+//                            fp32 1.08 to 1.46 up to beam 256, 0.92 to 1.09 beyond
+// At 2,048 queries a warp each fills the chip (2*10^5 x 128 u8, R = 32, beam 64 / 192): 651 / 1,317 us against
+// 659 / 1,593.  Bound: the chain of steps (row, gather, six barriers).
 #include <algorithm>
 
 #include "rr_common.cuh"
@@ -276,9 +281,11 @@ rr_status launch_t(const SearchArgs &a, cudaStream_t st) {
 
 // The CTA form: exact traversal, one parent per visit, no exact counters (its evaluation counts would differ), an
 // early stop that the lookahead can foresee, and beams long enough to have points in line (beam 16: 172 -> 186 us,
-// beam 64: 521 -> 400 us at 64 queries).
-bool beam_cta(const SearchArgs &a) {
-    return a.nq <= kBeamCta2 && a.beam >= kBeamCtaBeam && a.expand <= 1 && !a.count_bits && !a.stats && a.prec == RR_PREC_EXACT &&
+// beam 64: 521 -> 400 us at 64 queries).  With two warps a query only beams that these merge as fast as one warp does
+// (table above).
+bool beam_cta(const SearchArgs &a, int dtype_code) {
+    return a.nq <= (a.beam <= (dtype_code == DT_F32 ? kBeamCta2F32 : kBeamCta2Int) ? kBeamCta2 : kBeamCta4) &&
+           a.beam >= kBeamCtaBeam && a.expand <= 1 && !a.count_bits && !a.stats && a.prec == RR_PREC_EXACT &&
            (!a.use_es || a.es_metric == RR_ES_VISITED || a.es_metric == RR_ES_TOP1);
 }
 

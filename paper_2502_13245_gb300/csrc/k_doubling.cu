@@ -782,7 +782,9 @@ __global__ void zero_words_kernel(uint32_t *p, int64_t n) {
 }
 
 // Two CTAs of 256 threads (111 registers) fit an SM: up to two waves of them a round goes by CTA.  With more active
-// queries a warp each fills the chip, and the evaluations made for nothing would cost throughput.  Exact counters
+// queries a warp each fills the chip, and the evaluations made for nothing would cost throughput.  At the limit the
+// phase is still 2.1 times (fp32 2 KB, R = 128: 32.0 -> 15.1 ms) to 2.8 times faster (u8 128 B, R = 128: 17.1 -> 6.2; fp32
+// 800 B, R = 64: 21.0 -> 7.5); at 40 queries 2.4 to 3.0 times.  Exact counters
 // (stats) are kept by the warp form only: rr_query_stats.evals is what was evaluated, and the lookahead evaluates more.
 constexpr int kCtaRounds = 608;
 

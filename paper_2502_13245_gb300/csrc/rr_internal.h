@@ -184,7 +184,8 @@ void slack_coefficients(const rr_index *ix, int prec, float *A, float *Bq, float
 // k_beam_cta.cu
 constexpr int64_t kBeamCta8 = 304, kBeamCta4 = 608, kBeamCta2 = 1216;  // most queries with 8, 4, 2 warps each
 constexpr int kBeamCtaBeam = 32;                                       // the shortest beam
-bool beam_cta(const SearchArgs &a);
+constexpr int kBeamCta2Int = 128, kBeamCta2F32 = 256;                  // the longest with 2 warps: 8-bit, fp32
+bool beam_cta(const SearchArgs &a, int dtype_code);
 rr_status launch_beam_cta(const SearchArgs &a, cudaStream_t st, int dtype_code);
 rr_status launch_beam(const SearchArgs &a, int warps_per_cta, cudaStream_t s, int dtype_code);
 // Alg. 1 without early stop or range filter for graph construction: the queries are stored rows

@@ -373,3 +373,20 @@ def test_doubling_rounds_by_a_warp_per_query(rr, variant, kind):
         for g, w in zip(got.query(i), want.query(i % 50)):
             assert np.array_equal(g, w), i
     gi.close()
+
+
+@pytest.mark.parametrize("dtype,beam,nq,form", [
+    ("u8", 128, 609, "beam_cta"), ("u8", 128, 1216, "beam_cta"), ("u8", 129, 608, "beam_cta"), ("u8", 129, 609, "beam_warp"),
+    ("f32", 256, 1216, "beam_cta"), ("f32", 257, 608, "beam_cta"), ("f32", 257, 609, "beam_warp")])
+def test_limits_of_the_cta_form(rr, dtype, beam, nq, form):
+    """Two warps a query are the slower form for long beams; either side of each limit against the oracle."""
+    X, adj, Q = _data(1500, 12, 32, 64, 12)
+    r = _radius(X, Q, 12)
+    X, Q = X.astype(np.uint8 if dtype == "u8" else np.float32), Q.astype(np.uint8 if dtype == "u8" else np.float32)
+    gi, oi = rr.Index.from_arrays(X, adj, 0), oracle.Index(X, adj, 0)
+    o_ids, o_d, _ = oracle.range_search(oi, Q, r, "greedy", beam=beam, threads=os.cpu_count() or 4)
+    before = rr.rr_debug_count(form)
+    res = gi.range_search(np.tile(Q, (20, 1))[:nq], r, "greedy", beam=beam)
+    assert rr.rr_debug_count(form) == before + 1
+    _tiled(res, nq, o_ids, o_d)
+    gi.close()
