@@ -54,6 +54,14 @@ def log(*a):
     print("[bench]", *a, file=sys.stderr, flush=True)
 
 
+def emit(line, sweep):
+    """The result as one line on stdout.  The sweep it was chosen from has hundreds of entries: each goes to stderr, so
+    that the line stays short enough to be read from the end of a log."""
+    for s in sweep:
+        log("sweep", json.dumps({k: (round(v, 5) if isinstance(v, float) else v) for k, v in s.items()}))
+    print(json.dumps(line), flush=True)
+
+
 def dist_env():
     ws = int(os.environ.get("WORLD_SIZE", "1"))
     rank = int(os.environ.get("RANK", "0"))
@@ -825,9 +833,8 @@ def main():
             "gpu_launches": launches,
             "clocks": clocks,
             "cpu_baseline": cpu,
-            "sweep": [{k: (round(v, 5) if isinstance(v, float) else v) for k, v in s.items()} for s in sweep],
         }
-        print(json.dumps(line), flush=True)
+        emit(line, sweep)
     if ws > 1:
         torch.distributed.destroy_process_group()
 
