@@ -21,9 +21,9 @@
 // One pass: a match is appended to the item list as (query, key), counted in a
 // register of the thread that owns the query; the output's bin sort takes the
 // list.  The former form computed every distance twice with dp4a (count, then
-// fill): 1,000 queries x 2*10^6 x 256 bytes, 31.6 -> 3.7 ms; 2,000 x 5*10^5 x 256,
-// 15.8 -> 3.0 ms before the second epilogue group (GB300).  Bound: the producers'
-// and the epilogue's instructions; the tensor pipe is busy a tenth of the time.
+// fill): 1,000 queries x 2*10^6 x 256 bytes, 31.6 -> 3.7 ms (GB300).  Bound: the
+// producers' and the epilogue's instructions; the tensor pipe is busy a tenth of
+// the time.
 #include <cuda_fp16.h>
 
 #include <algorithm>

@@ -390,3 +390,17 @@ def test_limits_of_the_cta_form(rr, dtype, beam, nq, form):
     assert rr.rr_debug_count(form) == before + 1
     _tiled(res, nq, o_ids, o_d)
     gi.close()
+
+
+@pytest.mark.parametrize("dtype", ["u8", "f32"])
+def test_last_large_queries_are_handed_over(rr, dtype):
+    """Six queries with 50,000 results each: frontiers of thousands while the rest of the chip is idle go to the level
+    kernels, which end the phase."""
+    X, adj, live, Q = _all_in_range(60_000, 50_000, 24, 6, 13)
+    X, Q = (X, Q) if dtype == "u8" else (X.astype(np.float32), Q.astype(np.float32))
+    gi = rr.Index.from_arrays(X, adj, 0)
+    before = [rr.rr_debug_count("greedy_" + k) for k in ("handed", "levels")]
+    res = gi.range_search(Q, 1e9, "greedy", beam=16)
+    assert [rr.rr_debug_count("greedy_" + k) for k in ("handed", "levels")] == [before[0] + 6, before[1]]
+    _check_all(res, X, live, Q)
+    gi.close()
