@@ -487,11 +487,19 @@ rr_status run_bfs(Search &S, BfsShape shape, int32_t *np2, GreedyOut &go) {
         shape.clusters = (int)std::min<int64_t>(full, queued);
         hand = hand_bytes(queued, &pend_cap, &off_pk, &off_ps);
     }
-    int64_t want = std::min<int64_t>(result_cap(S, queued), known ? (int64_t)1 << 22 : (int64_t)1 << 20) + slack;
-    if ((s = grow(ix->item_key, (size_t)want * 8, 0, S.st)) != RR_OK) return s;
-    if ((s = grow(ix->item_slot, (size_t)want * 4, 0, S.st)) != RR_OK) return s;
+    auto grow_list = [&](int64_t entries) {
+        const rr_status e = grow(ix->item_key, (size_t)entries * 8, 0, S.st);
+        return e == RR_OK ? grow(ix->item_slot, (size_t)entries * 4, 0, S.st) : e;
+    };
+    const int64_t least = std::min<int64_t>(result_cap(S, queued), (int64_t)1 << 20) + slack;
+    s = grow_list(known ? std::min<int64_t>(result_cap(S, queued), (int64_t)1 << 22) + slack : least);
+    if (s == RR_ENOMEM && known) s = grow_list(least);
+    if (s != RR_OK) return s;
     if ((s = grow(ix->front, shape.clusters * front1, 0, S.st)) == RR_OK) s = grow(ix->hand, hand, 0, S.st);
     if (s == RR_ENOMEM) {  // the level kernels need a bitmap a query, no more
+        RR_CUDA(cudaStreamSynchronize(S.st));
+        grow_free(ix->front);
+        grow_free(ix->hand);
         if (!known && (s = read_queued(S, np2)) != RR_OK) return s;
         bool capped;
         return *np2 > 0 ? run_greedy(S, *np2, nullptr, go, &capped) : RR_OK;
@@ -540,9 +548,8 @@ rr_status run_bfs(Search &S, BfsShape shape, int32_t *np2, GreedyOut &go) {
         capped = S.hc[kCtrOverflow] != 0 || results > result_cap(S, *np2);  // a run that stopped: overflow
         if (capped || tail <= g.cap) break;
         // queries that this run handed over may be expanded further by the next
-        want = std::min<int64_t>(S.hc[kCtrPend + 1] > 0 ? 2 * results : results, result_cap(S, *np2)) + slack;
-        if ((s = grow(ix->item_key, (size_t)want * 8, 0, S.st)) != RR_OK) return s;
-        if ((s = grow(ix->item_slot, (size_t)want * 4, 0, S.st)) != RR_OK) return s;
+        const int64_t want = S.hc[kCtrPend + 1] > 0 ? 2 * results : results;
+        if ((s = grow_list(std::min<int64_t>(want, result_cap(S, *np2)) + slack)) != RR_OK) return s;
         RR_CUDA(cudaMemsetAsync(S.counters + kCtrBfsNext, 0, (kCtrWords - kCtrBfsNext) * 4, S.st));
         note_form(kFormClusterAgain);
     }

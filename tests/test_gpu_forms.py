@@ -404,3 +404,22 @@ def test_last_large_queries_are_handed_over(rr, dtype):
     assert [rr.rr_debug_count("greedy_" + k) for k in ("handed", "levels")] == [before[0] + 6, before[1]]
     _check_all(res, X, live, Q)
     gi.close()
+
+
+def test_a_device_without_room_for_the_clusters(rr):
+    """An index whose frontier lists are large (1 MB a cluster): without room for the larger item list the smaller one
+    serves; without room for the lists or the hand-over the level kernels do, and what was taken is given back."""
+    X, adj, live, Q = _all_in_range(200_000, 300, 12, 400, 14)
+    for nth, form in ((1, "greedy_cluster"), (2, "greedy_cluster"), (3, "greedy_levels"), (4, "greedy_levels")):
+        gi = rr.Index.from_arrays(X, adj, 0)
+        before = rr.rr_debug_count(form)
+        try:
+            rr.rr_debug_set("fail_alloc_after", nth)
+            res = gi.range_search(Q, 1e9, "greedy", beam=8)
+        finally:
+            rr.rr_debug_set("fail_alloc_after", -1)
+        assert rr.rr_debug_count(form) == before + 1, nth
+        _check_all(res, X, live, Q)
+        if form == "greedy_levels":  # no frontier list is held
+            assert rr.rr_index_info_get(gi.h).scratch_bytes < 152 << 20
+        gi.close()
