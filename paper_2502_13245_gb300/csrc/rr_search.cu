@@ -420,11 +420,11 @@ rr_status take_outgrown(Search &S, const BfsArgs &g, const SlotList &out, HandOv
     rr_index *ix = S.ix;
     rr_status s;
     int64_t most = ho.count;
-    std::vector<int32_t> count((size_t)out.n);
+    int32_t count[kBfsHandCap];
     for (int i = 0; i < out.n; i++)
-        RR_CUDA(cudaMemcpyAsync(&count[(size_t)i], S.slot_count + out.slot1[i] - 1, 4, cudaMemcpyDeviceToHost, S.st));
+        RR_CUDA(cudaMemcpyAsync(count + i, S.slot_count + out.slot1[i] - 1, 4, cudaMemcpyDeviceToHost, S.st));
     RR_CUDA(cudaStreamSynchronize(S.st));
-    for (int32_t c : count) most += c;
+    for (int i = 0; i < out.n; i++) most += count[i];
     const size_t off = ru((size_t)most * 8);
     if ((s = grow(ix->outgrown, off + (size_t)most * 4, 0, S.st)) != RR_OK) return s;
     uint64_t *key = (uint64_t *)ix->outgrown.p;
